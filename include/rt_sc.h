@@ -354,7 +354,11 @@ rt_status rt_get_stats(rt_grid g, rt_stats *out);
  * 3 = pipelined: chi and S staged one plane ahead by asynchronous copies, strip
  * edges exchanged through distributed shared memory).  Automatic choice:
  * variant 3 for RT_PREC_MIXED, 1 for FP64; rays per group and strips from the
- * runtime's count of co-resident clusters (rt_autotune measures instead).
+ * runtime's count of co-resident clusters and a cost model (rt_autotune measures
+ * instead).  Variant 3, and FP64's automatic choice, take the segment weights
+ * from a table of two values per ray and cell, filled once per medium and plan
+ * and kept by the grid, where that takes at most a quarter of the free device
+ * memory, and form them as they sweep otherwise.
  * Results do not depend on the configuration beyond rounding order.
  * Errors: RT_ERR_ARG for out-of-range values or no feasible configuration. */
 rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas, int threads,

@@ -266,6 +266,11 @@ struct rt_grid_s {
   // sweep plan
   int apg = 0, amax = 1, cluster = 1, threads = 256, slots = 1, variant = 1;
   size_t smem = 0;
+  // the streamed sweep (rt_stream.cu) takes the plan's place of variant 3, and of
+  // FP64's automatic variant 1, while the grid holds a weight table: `threads` are
+  // its threads, ncomp those with cells, depth its S ring
+  bool stream = false;
+  int depth = 0, ncomp = 0, one_pass = 0;
   int req_apg = 0, req_cluster = 0, req_threads = 0, req_variant = 0;
   std::vector<GroupParam> groups;
   std::vector<int> group_angles;   // angle index per AngleParam slot
@@ -365,8 +370,9 @@ struct rt_grid_s {
   std::vector<Graph> graphs;
   long long gen = 0;                  // bumped whenever a captured pointer or plan may change
   bool graphs_ok = true;              // false once a capture failed on this grid
-  // FP64 grids, one-cell-per-thread sweep: E and Psi0 per ray slot and cell,
-  // [2][slots][nf][cells], tabulated for the medium and plan of generation wt_gen
+  // segment weights E and Psi0 per ray slot and cell, tabulated for the medium and
+  // plan of generation wt_gen: the streamed sweep's interleaved table, or (FP64
+  // one-cell-per-thread sweep) [2][slots][nf][cells]
   void *wt = nullptr;
   size_t wt_bytes = 0;
   long long wt_gen = -1;
@@ -455,6 +461,7 @@ void build_rays(rt_grid g) {
 
 // Largest dynamic shared memory a sweep CTA may use.
 constexpr size_t kSweepSmemBudget = 200 * 1024;
+constexpr size_t kStreamSmemBudget = 224 * 1024;
 constexpr int kSMs = 152;
 
 int amax_for(int apg) { return apg <= 1 ? 1 : (apg <= 2 ? 2 : (apg <= 4 ? 4 : 8)); }
@@ -610,11 +617,138 @@ void split_last_wave(rt_grid g) {
   g->groups.swap(keep);
 }
 
+bool external_faces(rt_grid g) {
+  return g->desc.bc_lo[2] == RT_BC_EXTERNAL || g->desc.bc_hi[2] == RT_BC_EXTERNAL;
+}
+
+// Threads, shared memory and S-ring depth of a streamed-sweep CTA for `slots` rays
+// and C strips; false if it does not fit.
+struct StreamShape {
+  int threads = 0, ncomp = 0, depth = 0, tasks = 0, passes = 0;
+  size_t smem = 0;
+};
+bool stream_shape(rt_grid g, int slots, int C, StreamShape *out) {
+  const bool f64 = g->desc.prec == RT_PREC_FP64;
+  StreamShape sh;
+  int elems = 0;   // halo cells and halo-row segments, at most one of each a thread
+  auto over_axes = [&](auto fn) {
+    for (int a = 0; a < 3; ++a) {
+      if (!g->used_axis[a]) continue;
+      int cax[3];
+      rtk::plane_axes(a, cax);
+      fn(g->d.n[cax[0]], (g->d.n[cax[1]] + C - 1) / C);
+    }
+  };
+  over_axes([&](int Nu, int Rmax) {
+    sh.tasks = std::max(sh.tasks, f64 ? rtk::stream_tasks<double>(Nu, Rmax) : rtk::stream_tasks<float>(Nu, Rmax));
+    elems = std::max({elems, slots * (Rmax + 2), slots * (f64 ? rtk::stream_tasks<double>(Nu, 1) : rtk::stream_tasks<float>(Nu, 1))});
+  });
+  const int cap = f64 ? rtk::stream_max_threads<double, false>() : rtk::stream_max_threads<float, false>();
+  sh.passes = std::max(1, (sh.tasks + cap - 1) / cap);
+  const int per = (sh.tasks + sh.passes - 1) / sh.passes;
+  sh.ncomp = std::max(32, std::min(cap, ((per + 31) / 32) * 32));
+  if (g->req_threads > 0) sh.ncomp = std::min(g->req_threads, cap);
+  sh.threads = std::max(sh.ncomp, (elems + 31) / 32 * 32);
+  if (elems > rtk::stream_max_threads<float, true>()) return false;
+  for (int depth : {6, 4, 3}) {   // copies 4, 2 or 1 planes ahead
+    sh.depth = depth;
+    sh.smem = 0;
+    over_axes([&](int Nu, int Rmax) {
+      sh.smem = std::max(sh.smem, f64 ? rtk::stream_smem<double>(Nu, Rmax, slots, depth, false)
+                                      : rtk::stream_smem<float>(Nu, Rmax, slots, depth, true));
+    });
+    if (sh.smem <= (depth == 6 ? 48 : 100) * 1024) break;
+  }
+  if (sh.smem > kStreamSmemBudget) return false;
+  *out = sh;
+  return true;
+}
+
+int stream_resident(rt_grid g, const StreamShape &sh, int C) {
+  return g->desc.prec == RT_PREC_FP64
+             ? rtk::stream_max_active_clusters<double>(g->d, sh.tasks <= sh.ncomp, C, sh.threads, sh.smem)
+             : rtk::stream_max_active_clusters<float>(g->d, sh.tasks <= sh.ncomp, C, sh.threads, sh.smem);
+}
+
+// Plan of the streamed sweep: rays per group and strips per plane of the smallest
+// estimated time.  False where the grid does not stream (second order, subdomain
+// faces, an explicitly requested other variant, no memory for the table) or no
+// configuration fits.
+bool plan_stream(rt_grid g) {
+  const bool f64 = g->desc.prec == RT_PREC_FP64;
+  if (g->interp != RT_INTERP_LINEAR || g->wt_off || external_faces(g)) return false;
+  if (!(g->req_variant == 3 || g->req_variant == 0)) return false;
+  int minNv = 1 << 30;
+  for (int a = 0; a < 3; ++a) {
+    if (!g->used_axis[a]) continue;
+    int cax[3];
+    rtk::plane_axes(a, cax);
+    minNv = std::min(minNv, g->d.n[cax[1]]);
+  }
+  int depth_max = 1;   // planes of the longest sweep
+  for (int a = 0; a < 3; ++a)
+    if (g->used_axis[a]) depth_max = std::max(depth_max, g->d.n[a]);
+  double best = 1e300;
+  int bapg = 0, bC = 0;
+  for (int apg = 1; apg <= rtk::kStreamRays; ++apg) {
+    if (g->req_apg > 0 && apg != g->req_apg) continue;
+    std::vector<GroupParam> gr;
+    std::vector<int> ga;
+    int namax = 0;
+    make_groups(g, apg, gr, ga, &namax);
+    const long long clusters = (long long)gr.size() * g->d.nf;
+    for (int C = 1; C <= std::min(16, minNv); ++C) {
+      if (g->req_cluster > 0 && C != g->req_cluster) continue;
+      StreamShape sh;
+      if (!stream_shape(g, namax, C, &sh)) continue;
+      int nres = stream_resident(g, sh, C);
+      if (nres <= 0) nres = 1;
+      // microseconds a sweep.  A plane costs the CTA about 1 us (its barrier, halo and
+      // stores) and each thread's row segments passes x rays; a ray's share is latency
+      // (0.25 us) until the SM's warps fill the issue slots (0.033 us a warp; float64:
+      // the FP64 pipe, 0.2 us a warp).  Fitted to sweeps of 32^3 to 256^3 and 2D grids,
+      // 1 to 7 rays a group and 1 to 16 strips: within 15 %.
+      const double waves = std::ceil((double)clusters / nres);
+      const double share = std::max(1.0, std::ceil((double)std::min<long long>(clusters, nres) * C / kSMs));
+      const double warps = share * (sh.ncomp / 32);
+      const double ray = f64 ? std::max(0.3, 0.2 * warps) : std::max(0.25, 0.033 * warps);
+      const double step = (share > 1.0 ? 1.3 : 1.0) + sh.passes * (0.4 + namax) * ray;
+      // every group's partial of J, written here and read by the update, at 5 TB/s
+      const double partials = (double)gr.size() * (double)N_of(g) * g->tsize * 2.0 / 5e6;
+      const double est = waves * depth_max * step + partials;
+      if (est < best * 0.999) {
+        best = est;
+        bapg = apg;
+        bC = C;
+      }
+    }
+  }
+  if (!bapg) return false;
+  int namax = 0;
+  StreamShape sh;
+  make_groups(g, bapg, g->groups, g->group_angles, &namax);
+  if (!stream_shape(g, namax, bC, &sh)) return false;
+  g->stream = true;
+  g->variant = f64 && g->req_variant == 0 ? 1 : 3;
+  g->apg = bapg;
+  g->slots = namax;
+  g->amax = amax_for(namax);
+  g->cluster = bC;
+  g->threads = sh.threads;
+  g->depth = sh.depth;
+  g->ncomp = sh.ncomp;
+  g->one_pass = sh.tasks <= sh.ncomp;
+  g->smem = sh.smem;
+  return true;
+}
+
 // Choose rays per group and strips per plane: the estimated sweep time is
 // (waves of resident clusters) x (rays per group) x (cells per strip) x
 // (CTAs sharing an SM), from the runtime's count of co-resident clusters
 // (clusters cannot straddle a GPC, so this is not simply SMs / C).
 void plan_groups(rt_grid g) {
+  g->stream = false;
+  if (plan_stream(g)) return;
   int minNv = 1 << 30;
   for (int a = 0; a < 3; ++a) {
     if (!g->used_axis[a]) continue;
@@ -845,7 +979,13 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
   A.write_ghosts = 1;
   A.skip_if_done = 1;
   A.cluster = g->cluster;
-  const bool wt = g->wt && g->wt_gen == g->gen && g->variant == 1 && g->interp == RT_INTERP_LINEAR;
+  const bool ready = g->wt && g->wt_gen == g->gen;
+  A.WT = ready && g->stream ? (const T *)g->wt : nullptr;
+  A.wt_slot = (long long)rtk::stream_slot_elems<T>(g->d, g->used_axis);
+  A.depth = g->depth;
+  A.ncomp = g->ncomp;
+  A.one_pass = g->one_pass;
+  const bool wt = ready && !g->stream && g->variant == 1 && g->interp == RT_INTERP_LINEAR;
   const size_t half = g->wt_bytes / 2;
   A.WE = wt ? (const T *)g->wt : nullptr;
   A.WP = wt ? (const T *)((const char *)g->wt + half) : nullptr;
@@ -860,33 +1000,45 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
   return A;
 }
 
-// The one-cell-per-thread sweep of FP64 grids reads its segment weights E, Psi0
-// (functions of chi alone) from a table filled once per medium and plan: the
-// FP64 exponential and divide are then paid once, not every formal solution.
-// Without the memory for it, the sweep computes them as before.
+// The segment weights E, Psi0 are functions of chi alone: the streamed sweep, and
+// the one-cell-per-thread sweep of FP64 grids, read them from a table filled once
+// per medium and plan.  A table takes at most a quarter of the free device memory;
+// without the room the grid is planned without it (the sweeps then compute the
+// weights as they go).
 template <typename T>
 rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
-  if (sizeof(T) != 8 || g->variant != 1 || g->interp != RT_INTERP_LINEAR || g->wt_off) return RT_OK;
+  if (g->wt_off || !(g->stream || (sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR))) return RT_OK;
   if (g->wt && g->wt_gen == g->gen) return RT_OK;
-  const size_t need = 2 * g->group_angles.size() * (size_t)N_of(g) * sizeof(T);
+  const size_t slots = g->group_angles.size();
+  const size_t need = g->stream ? slots * g->d.nf * rtk::stream_slot_elems<T>(g->d, g->used_axis) * sizeof(T)
+                                : 2 * slots * (size_t)N_of(g) * sizeof(T);
   if (need > g->wt_bytes) {
     if (g->wt) cudaFree(g->wt);
     g->wt = nullptr;
     g->wt_bytes = 0;
-    if (cudaMalloc(&g->wt, need) != cudaSuccess) {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || (g->stream && need > fr / 4) ||
+        cudaMalloc(&g->wt, need) != cudaSuccess) {
       cudaGetLastError();
       g->wt = nullptr;
       g->wt_off = true;
-      return RT_OK;
+      if (!g->stream) return RT_OK;
+      plan_groups(g);
+      return upload_plan<T>(g);
     }
     g->wt_bytes = need;
     g->gen++;   // a new buffer: captured graphs must not replay the old pointers
   }
   rtk::SweepArgs<T> A = sweep_args<T>(g);
-  T *WE = (T *)g->wt, *WP = (T *)((char *)g->wt + g->wt_bytes / 2);
-  for (size_t gi = 0; gi < g->groups.size(); ++gi) {
-    CU(rtk::launch_seg_table<T>(A, (int)gi, g->groups[gi].na, WE, WP, s));
+  if (g->stream) {
+    CU(rtk::launch_stream_table<T>(A, (T *)g->wt, s));
     g->launches++;
+  } else {
+    T *WE = (T *)g->wt, *WP = (T *)((char *)g->wt + g->wt_bytes / 2);
+    for (size_t gi = 0; gi < g->groups.size(); ++gi) {
+      CU(rtk::launch_seg_table<T>(A, (int)gi, g->groups[gi].na, WE, WP, s));
+      g->launches++;
+    }
   }
   g->wt_gen = g->gen;
   return RT_OK;
@@ -905,7 +1057,10 @@ rt_status enqueue_sweep(rt_grid g, rtk::SweepArgs<T> &A, bool moments, cudaStrea
     CU(cudaEventCreate(&p.b));
     CU(cudaEventRecord(p.a, s));
   }
-  if (g->interp == RT_INTERP_QUADRATIC) {
+  if (g->stream && !A.WT) return fail(RT_ERR_STATE, "streamed sweep without its weight table");
+  if (g->stream) {
+    CU(rtk::launch_sweep_stream<T>(A, moments, g->threads, g->smem, s));
+  } else if (g->interp == RT_INTERP_QUADRATIC) {
     CU(rtk::launch_sweep_quad<T>(A, g->amax, moments, g->threads, g->smem, s));
   } else if (g->variant == 3) {
     CU(rtk::launch_sweep_pipe<T>(A, g->amax, moments, g->threads, g->smem, s));
@@ -1049,8 +1204,8 @@ void solve_args(rt_grid g, int incremental, bool gs, rtk::SweepArgs<T> &A, rtk::
   A = sweep_args<T>(g);
   A.incremental = incremental;
   int nxg = 0;
-  if (sizeof(T) == 4 && !gs && g->variant == 3 && g->interp == RT_INTERP_LINEAR && g->d.n[0] % 4 == 0 &&
-      g->d.n[1] % 4 == 0) {
+  if (sizeof(T) == 4 && !gs && g->variant == 3 && g->interp == RT_INTERP_LINEAR &&
+      (A.WT || (g->d.n[0] % 4 == 0 && g->d.n[1] % 4 == 0))) {
     while (nxg < (int)g->groups.size() && g->groups[nxg].axis == 0) ++nxg;
     A.jx = 1;
   }
@@ -1129,13 +1284,15 @@ rt_status ali_loop(rt_grid g, const rt_solve_opts *opts, cudaStream_t s, int *it
   const bool gs = g->iteration == RT_ITER_GAUSS_SEIDEL && !g->lte;
   const int incremental = (g->desc.prec == RT_PREC_MIXED && g->interp == RT_INTERP_LINEAR) ? 1 : 0;
   rtk::GsArgs<T> GA{};
-  if (gs) {
-    rt_status r = gs_setup<T>(g, s, incremental != 0, GA);
+  {
+    rt_status r = ensure_seg_table<T>(g, s);   // (without the room for a table this replans)
     if (r != RT_OK) return r;
   }
-  {
-    rt_status r = ensure_seg_table<T>(g, s);
+  if (gs) {
+    const long long gen = g->gen;
+    rt_status r = gs_setup<T>(g, s, incremental != 0, GA);
     if (r != RT_OK) return r;
+    if (g->wt_gen == gen) g->wt_gen = g->gen;   // new buffers of its own leave the table as it was
   }
   rtk::SweepArgs<T> A;
   rtk::AliArgs<T> L;
@@ -1357,6 +1514,8 @@ rt_status formal_once(rt_grid g, cudaStream_t s) {
 
 template <typename T>
 rt_status moments_sweep(rt_grid g, cudaStream_t s) {
+  rt_status r0 = ensure_seg_table<T>(g, s);
+  if (r0 != RT_OK) return r0;
   const size_t need = g->groups.size();
   if (need > g->mpart_groups) {
     if (g->Mpart) cudaFree(g->Mpart);
@@ -1364,8 +1523,6 @@ rt_status moments_sweep(rt_grid g, cudaStream_t s) {
     CU(cudaMalloc(&g->Mpart, need * 9 * (size_t)N_of(g) * sizeof(T)));
     g->mpart_groups = need;
   }
-  rt_status r0 = ensure_seg_table<T>(g, s);
-  if (r0 != RT_OK) return r0;
   rtk::SweepArgs<T> A = sweep_args<T>(g);
   A.parity_offset = -1;
   A.write_ghosts = 0;
@@ -1485,7 +1642,11 @@ rt_status plan_first64(rt_grid g) {
     g->first64->shadow = true;
     // a few FP64 iterations per solve: their segment weights are tabulated per
     // medium when the table is modest (it holds E and Psi0 of every ray and cell)
-    g->first64->wt_off = 2.0 * g->na * (double)N_of(g) * 8.0 > kShadowTableMax;
+    if (2.0 * g->na * (double)N_of(g) * 8.0 > kShadowTableMax) {
+      g->first64->wt_off = true;
+      plan_groups(g->first64);
+      if ((r = upload_plan_any(g->first64)) != RT_OK) return r;
+    }
   }
   rt_status r = rt_set_opacity_source(g->first64, g->chi, g->eps, g->B, g->fw, 1);
   if (r != RT_OK) return r;
@@ -1686,12 +1847,14 @@ rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
               + 6 * D.nfreq * na * gsize * ts  // ghosts (two parities, increments) and inflow faces
               + groups * N * ts * 11           // J, Lambda* and moment partials
               + 8 * (16 * N + cells);          // moments outputs
-  if (D.prec == RT_PREC_FP64) b += 2 * na * N * 8;   // tabulated segment weights (one-cell sweep)
+  // tabulated segment weights: two values per ray and cell, rows padded to 16 bytes
+  const long long pad = std::max({(D.nx + 3) / 4 * 4 * (long long)D.ny * D.nz, D.nx * ((D.ny + 3) / 4 * 4LL) * D.nz});
+  b += 2 * na * pad * D.nfreq * ts;
   // a mixed grid's internal FP64 grid for its FP64 iterations: fields, FP64
   // copies, ghosts, J partials (no moments pass, no table)
   if (D.prec == RT_PREC_MIXED) {
     b += 8 * N * 11 + 8 * N * 6 + 6 * D.nfreq * na * gsize * 8 + groups * N * 8;
-    if (2.0 * na * (double)N * 8.0 <= kShadowTableMax) b += 2 * na * N * 8;   // its segment-weight table
+    if (2.0 * na * (double)N * 8.0 <= kShadowTableMax) b += 2 * na * pad * D.nfreq * 8;   // its segment-weight table
   }
   *bytes = b;
   return RT_OK;
@@ -2411,6 +2574,12 @@ namespace {
 
 bool ls_mergeable(const LsMember *x) { return x->g->variant == 3; }
 
+template <typename T>
+bool ls_streams(const LsMember *x) {
+  if constexpr (sizeof(T) == 4) return x->Af.WT != nullptr;
+  else return x->Ad.WT != nullptr;
+}
+
 // shared launches of the pipelined sweeps of members `idx` (one precision)
 template <typename T>
 rt_status ls_sweep_shared(rt_lockstep L, const std::vector<LsMember *> &idx) {
@@ -2421,11 +2590,14 @@ rt_status ls_sweep_shared(rt_lockstep L, const std::vector<LsMember *> &idx) {
     const rt_grid g0 = idx[i]->g;
     // (rows of every sweep axis a multiple of 4 cells: the float32 kernel's 128-bit rows)
     const bool v0 = sizeof(T) == 4 && g0->d.n[0] % 4 == 0 && g0->d.n[1] % 4 == 0;
+    const bool st0 = ls_streams<T>(idx[i]);
     std::vector<LsMember *> set;
     for (size_t j = i; j < idx.size(); ++j) {
       const rt_grid gj = idx[j]->g;
       const bool vj = sizeof(T) == 4 && gj->d.n[0] % 4 == 0 && gj->d.n[1] % 4 == 0;
-      if (!used[j] && gj->cluster == g0->cluster && vj == v0) {
+      const bool stj = ls_streams<T>(idx[j]);
+      if (!used[j] && gj->cluster == g0->cluster && stj == st0 &&
+          (st0 ? rtk::stream_ragged<T>(gj->d) == rtk::stream_ragged<T>(g0->d) : vj == v0)) {
         used[j] = true;
         set.push_back(idx[j]);
       }
@@ -2449,7 +2621,8 @@ rt_status ls_sweep_shared(rt_lockstep L, const std::vector<LsMember *> &idx) {
         x->g->launches++;
         if (M.n > 1) x->g->stats.shared_launches++;
       }
-      CU(rtk::launch_sweep_multi<T>(M, amax, threads, smem, L->s));
+      CU(st0 ? rtk::launch_stream_multi<T>(M, threads, smem, L->s)
+             : rtk::launch_sweep_multi<T>(M, amax, threads, smem, L->s));
       L->shared++;
     }
   }

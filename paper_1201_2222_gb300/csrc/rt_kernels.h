@@ -31,6 +31,12 @@ struct SweepArgs {
   int ray_slots;             // shared-memory planes per ray slot (>= rays of any group)
   const T *WE, *WP;          // one-cell-per-thread sweep: E and Psi0 per ray slot and cell,
                              // [slot][nf][w][v][u] of the slot's group (NULL: computed)
+  const T *WT;               // streamed sweep: E and Psi0 interleaved per row segment, [slot][nf][wt_slot]
+                             //    (NULL: not streamed)
+  long long wt_slot;         //    elements per ray slot and frequency
+  int depth;                 //    planes of a CTA's S ring: 3, 4 or 6
+  int ncomp;                 //    its threads with cells
+  int one_pass;              //    1: a strip's row segments are at most ncomp
   int gs_forward;            // 1: Gauss-Seidel forward phase -- groups crossing the
   int gs_axis;               //    gs_axis face with mu < 0 (the reverse rays) do nothing
   // subdomain (EXTERNAL) z faces, side 0 = low, 1 = high (one-cell-per-thread
@@ -147,6 +153,33 @@ struct MultiSweep {
 };
 template <typename T>
 cudaError_t launch_sweep_multi(const MultiSweep<T> &M, int amax, int threads, size_t smem, cudaStream_t s);
+// Streamed sweep (rt_stream.cu): at most kStreamRays rays per group and
+// stream_max_threads threads per CTA.  FP64 and the moments pass hold more per
+// thread: 384 threads leave them 168 registers.
+constexpr int kStreamRays = 8;
+template <typename T, bool MOM>
+constexpr int stream_max_threads() { return sizeof(T) == 8 || MOM ? 384 : 512; }
+constexpr int kStreamTimeout = 33;    // device error: a neighbouring strip's row did not arrive
+constexpr int kStreamPrefetch = 3;   // planes between the L2 prefetch of the weights and their use
+template <typename T>
+cudaError_t launch_sweep_stream(const SweepArgs<T> &A, bool moments, int threads, size_t smem, cudaStream_t s);
+template <typename T>
+cudaError_t launch_stream_multi(const MultiSweep<T> &M, int threads, size_t smem, cudaStream_t s);
+// E and Psi0 of every ray slot and cell into WT (A's groups and opacity copies)
+template <typename T>
+cudaError_t launch_stream_table(const SweepArgs<T> &A, T *WT, cudaStream_t s);
+template <typename T>
+int stream_max_active_clusters(const Dims &d, bool one_pass, int cluster, int threads, size_t smem);
+// shared memory of a CTA; row segments (tasks) of `rows` rows; table elements per
+// ray slot and frequency; whether rows of some axis are no multiple of a segment
+template <typename T>
+size_t stream_smem(int Nu, int Rmax, int slots, int depth, bool incremental);
+template <typename T>
+int stream_tasks(int Nu, int rows);
+template <typename T>
+size_t stream_slot_elems(const Dims &d, const int used_axis[3]);
+template <typename T>
+bool stream_ragged(const Dims &d);
 // cells per thread of the second-order sweep
 constexpr int kQuadSeg = 2;
 // second-order sweep (rt_quad.cu): monotonic quadratic face interpolation and
