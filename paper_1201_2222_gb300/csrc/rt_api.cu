@@ -1512,6 +1512,13 @@ rt_status formal_once(rt_grid g, cudaStream_t s) {
   return RT_OK;
 }
 
+// the groups (the first ones) whose moment partials are in their plane layout
+int x_groups(rt_grid g) {
+  int n = 0;
+  while (g->stream && n < (int)g->groups.size() && g->groups[n].axis == 0) ++n;
+  return n;
+}
+
 template <typename T>
 rt_status moments_sweep(rt_grid g, cudaStream_t s) {
   rt_status r0 = ensure_seg_table<T>(g, s);
@@ -1527,6 +1534,7 @@ rt_status moments_sweep(rt_grid g, cudaStream_t s) {
   A.parity_offset = -1;
   A.write_ghosts = 0;
   A.skip_if_done = 0;
+  A.jx = g->stream ? 1 : 0;
   return enqueue_sweep<T>(g, A, true, s, nullptr);
 }
 
@@ -2110,11 +2118,11 @@ rt_status rt_moments(rt_grid g, double *J, double *H, double *K, double *f, doub
   if ((r = permute_any(g, Ssrc, g->SP, s)) != RT_OK) return r;
   if (g->desc.prec == RT_PREC_FP64) {
     if ((r = moments_sweep<double>(g, s)) != RT_OK) return r;
-    CU(rtk::launch_reduce_moments<double>(g->d, (int)g->groups.size(), (const double *)g->Jpart,
+    CU(rtk::launch_reduce_moments<double>(g->d, (int)g->groups.size(), x_groups(g), (const double *)g->Jpart,
                                           (const double *)g->Mpart, dJ, dH, dK, dF, g->two_d, s));
   } else {
     if ((r = moments_sweep<float>(g, s)) != RT_OK) return r;
-    CU(rtk::launch_reduce_moments<float>(g->d, (int)g->groups.size(), (const float *)g->Jpart,
+    CU(rtk::launch_reduce_moments<float>(g->d, (int)g->groups.size(), x_groups(g), (const float *)g->Jpart,
                                          (const float *)g->Mpart, dJ, dH, dK, dF, g->two_d, s));
   }
   if (g->last_incremental) {

@@ -46,7 +46,7 @@ struct SweepArgs {
   int ext[2];
   const T *xchi[2], *xS[2], *xB[2], *xI[2];
   T *xout[2];
-  int jx;                    // 1: the float32 pipelined sweep writes the J partials of
+  int jx;                    // 1: the float32 pipelined sweep and the streamed one write the partials of
                              //    groups sweeping along x in their plane layout [x][z][y]
                              //    (contiguous rows); consumers must read them so
 };
@@ -228,9 +228,8 @@ cudaError_t launch_fill_bc(const Dims &d, int na, int face, int mode, const doub
 template <typename T>
 cudaError_t launch_reduce_J(const Dims &d, int ngroups, const T *Jpart, double *J, cudaStream_t s);
 template <typename T>
-cudaError_t launch_reduce_moments(const Dims &d, int ngroups, const T *Jpart, const T *Mpart,
-                                  double *J, double *H, double *K, double *F, int two_d,
-                                  cudaStream_t s);
+cudaError_t launch_reduce_moments(const Dims &d, int ngroups, int nxg, const T *Jpart, const T *Mpart,
+                                  double *J, double *H, double *K, double *F, int two_d, cudaStream_t s);
 // per frequency: the smallest eps among optically thick cells (1 - Lambda* < 1/2),
 // as the bits of a non-negative double (atomicMin); cells with none leave 1.0
 cudaError_t launch_eps_thick_min(const Dims &d, const double *eps, const double *oml,

@@ -773,17 +773,19 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
         for (int j = 0; j < SEG; ++j)
           if (!RAG || u0 + j < Nu) jp[j * jcol] = (j & 1) ? Jp[j / 2].y : Jp[j / 2].x;
       }
-      if (MOM) {
-        const long long canon = (long long)u0 * csu + (long long)(v0 + lv) * csv + (long long)plane_of(t) * csw;
-        T *M = A.Mpart + (long long)gi * 9 * A.d.nf * cells + (long long)f * cells;
+      if (MOM) {   // laid out as the J partials are
+        T *mp = A.Mpart + (long long)gi * 9 * A.d.nf * cells + (jp - (A.Jpart + (long long)gi * A.d.nf * cells));
         const long long qs = (long long)A.d.nf * cells;
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-          const V2 *src = q < 3 ? Hm[MOM ? q : 0] : Km[MOM ? q - 3 : 0];
+        for (int q = 0; q < 9; ++q, mp += qs) {
+          const V2(&src)[NP] = q < 3 ? Hm[MOM ? (q < 3 ? q : 0) : 0] : Km[MOM ? (q < 3 ? 0 : q - 3) : 0];
+          if (!RAG && jcol == 1) {
+            store_seg(mp, src);
+          } else {
 #pragma unroll
-          for (int j = 0; j < SEG; ++j)
-            if (!RAG || u0 + j < Nu)
-              M[q * qs + RT_IDX(canon + j * csu, cells, 82)] = (j & 1) ? src[j / 2].y : src[j / 2].x;
+            for (int j = 0; j < SEG; ++j)
+              if (!RAG || u0 + j < Nu) mp[j * jcol] = (j & 1) ? src[j / 2].y : src[j / 2].x;
+          }
         }
       }
     }
