@@ -1196,7 +1196,7 @@ rt_status gs_setup(rt_grid g, cudaStream_t s, bool incremental, rtk::GsArgs<T> &
 
 // Sweep and Jacobi-update arguments of an ALI solve of g with the pipelined or
 // one-cell-per-thread sweep (the Gauss-Seidel forward-phase flags are set by the
-// caller).  The float32 pipelined sweep writes the partials of the groups
+// caller).  The streamed and the float32 pipelined sweep write the partials of the groups
 // sweeping along x (the first groups) in their plane layout, which the Jacobi
 // update reads.
 template <typename T>
@@ -1204,8 +1204,8 @@ void solve_args(rt_grid g, int incremental, bool gs, rtk::SweepArgs<T> &A, rtk::
   A = sweep_args<T>(g);
   A.incremental = incremental;
   int nxg = 0;
-  if (sizeof(T) == 4 && !gs && g->variant == 3 && g->interp == RT_INTERP_LINEAR &&
-      (A.WT || (g->d.n[0] % 4 == 0 && g->d.n[1] % 4 == 0))) {
+  if (!gs && (A.WT || (sizeof(T) == 4 && g->variant == 3 && g->interp == RT_INTERP_LINEAR &&
+                       g->d.n[0] % 4 == 0 && g->d.n[1] % 4 == 0))) {
     while (nxg < (int)g->groups.size() && g->groups[nxg].axis == 0) ++nxg;
     A.jx = 1;
   }

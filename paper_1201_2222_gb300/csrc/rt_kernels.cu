@@ -1433,12 +1433,43 @@ __device__ __forceinline__ long long perm_index(const Dims &d, int a, long long 
 // A block owns a tile of 32 x 32 cells (x, y) of one z plane and frequency; the
 // sweep copies of the new S (or of dS) are written x-contiguous for the y and z
 // sweeps and through a shared-memory transpose, y-contiguous, for the x sweep.
+// The partials of the first nxg groups (sweeps along x) may be in the [x][z][y]
+// layout: they are summed where they lie and the sums transposed once.
+// Bound by memory in large grids and by the chain of its loads in small ones: the
+// loads of a thread's cells go out together, four groups at a time, and a grid of
+// few tiles (kAliWideBlocks: two a SM) takes one cell a thread instead of four.
+// 40 updates of 256^3 became 10.7 ms shorter, those of 8 boxes of 25^3 to 64^3
+// (1000 in all) 8.8 ms.
 constexpr int kAliTile = 32;
-constexpr int kAliRows = 8;
+constexpr int kAliRows = 8;                 // rows of threads a block, ordinary grids
+constexpr int kAliWideBlocks = 304;    // up to so many tiles: 32 rows of threads
 
+// The sum of a cell's partials in group order: FP64, or exact in a float pair
+// (TwoSum) with one FP64 add at the end -- the FP64 sum to ~1e-14 at FP32 cost.
 template <typename T>
-__global__ void __launch_bounds__(kAliTile * kAliRows) ali_update_kernel(const AliArgs<T> A) {
+struct PartSum;
+template <>
+struct PartSum<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float s2 = hi + v;
+    const float bp = s2 - hi;
+    lo += (hi - (s2 - bp)) + (v - bp);
+    hi = s2;
+  }
+  __device__ __forceinline__ double total() const { return (double)hi + (double)lo; }
+};
+template <>
+struct PartSum<double> {
+  double hi = 0.0;
+  __device__ __forceinline__ void add(double v) { hi += v; }
+  __device__ __forceinline__ double total() const { return hi; }
+};
+
+template <typename T, int ROWS>
+__global__ void __launch_bounds__(kAliTile * ROWS) ali_update_kernel(const AliArgs<T> A) {
   if (A.st->done) return;
+  constexpr int KR = kAliTile / ROWS;
   __shared__ T tile[kAliTile][kAliTile + 1];
   const int nx = A.d.n[0], ny = A.d.n[1], nz = A.d.n[2];
   const int tx = threadIdx.x % kAliTile, ty = threadIdx.x / kAliTile;
@@ -1446,74 +1477,62 @@ __global__ void __launch_bounds__(kAliTile * kAliRows) ali_update_kernel(const A
   const int x0 = (blockIdx.x % tiles_x) * kAliTile, y0 = (blockIdx.x / tiles_x) * kAliTile;
   const int z = blockIdx.y, f = blockIdx.z;
   const long long cells = A.d.cells;
-  const long long fbase = (long long)f * cells;
+  const long long fbase = (long long)f * cells, gstride = (long long)A.d.nf * cells;
   const bool first = A.st->iter == 0;
   const bool inc = A.incremental && !first;
   const int x = x0 + tx;
   double rmax = 0.0;
   float rmaxf = 0.f;   // float32 sweeps: the maximum of the quantities taken in float32
-  // float32 partials are summed exactly into a float pair (TwoSum) in group
-  // order; those of the first nxg groups (sweeps along x) are in the [x][z][y]
-  // layout and come through a shared-memory transpose of the tile
   if (A.fmask && A.fmask[f]) {   // this frequency is solved by another grid
     block_max_to(0.0, &A.st->resid_bits);
     return;
   }
-  constexpr int KR = kAliTile / kAliRows;
-  float xhi[KR], xlo[KR];
+  PartSum<T> sum[KR];
+  if (A.Jpart && A.nxg > 0) {
+    const T *src = A.Jpart + fbase + ((long long)(x0 + ty) * nz + z) * ny + y0 + tx;
+#pragma unroll 4
+    for (int p = 0; p < A.nxg; ++p, src += gstride) {
 #pragma unroll
-  for (int k = 0; k < KR; ++k) xhi[k] = xlo[k] = 0.f;
-  if (sizeof(T) == 4 && A.Jpart && A.nxg > 0) {
-    __shared__ float tJ[kAliTile][kAliTile + 1];
-    for (int p = 0; p < A.nxg; ++p) {
-      const float *src = reinterpret_cast<const float *>(A.Jpart) + ((long long)p * A.d.nf + f) * cells;
+      for (int k = 0; k < KR; ++k)
+        sum[k].add(x0 + ty + k * ROWS < nx && y0 + tx < ny ? src[(long long)k * ROWS * nz * ny] : T(0));
+    }
 #pragma unroll
-      for (int k = 0; k < KR; ++k) {
-        const int xx = x0 + ty + k * kAliRows, yy = y0 + tx;
-        tJ[ty + k * kAliRows][tx] = (xx < nx && yy < ny) ? src[((long long)xx * nz + z) * ny + yy] : 0.f;
-      }
+    for (int k = 0; k < KR; ++k) tile[ty + k * ROWS][tx] = sum[k].hi;
+    if constexpr (sizeof(T) == 4) {
+      __shared__ float low[kAliTile][kAliTile + 1];
+#pragma unroll
+      for (int k = 0; k < KR; ++k) low[ty + k * ROWS][tx] = sum[k].lo;
       __syncthreads();
 #pragma unroll
-      for (int k = 0; k < KR; ++k) {
-        const float v = tJ[tx][ty + k * kAliRows];
-        const float s2 = xhi[k] + v;
-        const float bp = s2 - xhi[k];
-        xlo[k] += (xhi[k] - (s2 - bp)) + (v - bp);
-        xhi[k] = s2;
-      }
+      for (int k = 0; k < KR; ++k) sum[k].lo = low[tx][ty + k * ROWS];
+    } else {
       __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < KR; ++k) sum[k].hi = tile[tx][ty + k * ROWS];
+    __syncthreads();   // the tile is written again below
+  }
+  const long long c0 = fbase + ((long long)z * ny + y0 + ty) * nx + x;   // cell of k: c0 + k ROWS nx
+  bool live[KR];
+#pragma unroll
+  for (int k = 0; k < KR; ++k) live[k] = x < nx && y0 + ty + k * ROWS < ny;
+  if (A.Jpart) {
+    const T *src = A.Jpart + c0 + A.nxg * gstride;
+#pragma unroll 4
+    for (int p = A.nxg; p < A.ngroups_per_f; ++p, src += gstride) {
+#pragma unroll
+      for (int k = 0; k < KR; ++k) sum[k].add(live[k] ? src[(long long)k * ROWS * nx] : T(0));
     }
   }
 #pragma unroll
   for (int k = 0; k < KR; ++k) {
-    const int y = y0 + ty + k * kAliRows;
+    const int y = y0 + ty + k * ROWS;
     T snew = T(0);
-    if (x < nx && y < ny) {
-      const long long c = ((long long)z * ny + y) * nx + x;
-      const long long i = fbase + c;
-      double dJ;
-      if (!A.Jpart) {
-        // the formal solution was done elsewhere (a mixed grid's FP64 first one):
-        // its J is already in J64
-        dJ = A.J64[i];
-      } else if (sizeof(T) == 4) {
-        // float32 partials summed exactly into a float pair (TwoSum), then one FP64
-        // add: the result is the FP64 sum to ~1e-14 at FP32 cost
-        float hi = xhi[k], lo = xlo[k];
-#pragma unroll 4
-        for (int p = A.nxg; p < A.ngroups_per_f; ++p) {
-          const float x = (float)A.Jpart[(long long)p * A.d.nf * cells + i];
-          const float s2 = hi + x;
-          const float bp = s2 - hi;
-          lo += (hi - (s2 - bp)) + (x - bp);
-          hi = s2;
-        }
-        dJ = (double)hi + (double)lo;
-      } else {
-        dJ = 0.0;
-#pragma unroll 4
-        for (int p = 0; p < A.ngroups_per_f; ++p) dJ += (double)A.Jpart[(long long)p * A.d.nf * cells + i];
-      }
+    if (live[k]) {
+      const long long i = c0 + (long long)k * ROWS * nx;
+      // no partials: the formal solution was done elsewhere (a mixed grid's FP64
+      // first one), its J is already in J64
+      const double dJ = A.Jpart ? sum[k].total() : A.J64[i];
       // incremental solves accumulate J in FP64 from the swept increments (an
       // FP64 iteration's J replaces the accumulated one)
       const double J = (inc && A.Jpart) ? A.J64[i] + dJ : dJ;
@@ -1569,14 +1588,14 @@ __global__ void __launch_bounds__(kAliTile * kAliRows) ali_update_kernel(const A
       if (A.SP[2]) A.SP[2][i] = snew;                                                 // [z][y][x]
       if (A.SP[1]) A.SP[1][fbase + ((long long)y * nz + z) * nx + x] = snew;          // [y][z][x]
     }
-    tile[ty + k * kAliRows][tx] = snew;
+    tile[ty + k * ROWS][tx] = snew;
   }
   if (A.SP[0]) {                                                                      // [x][z][y]
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kAliTile / kAliRows; ++k) {
-      const int xx = x0 + ty + k * kAliRows, yy = y0 + tx;
-      if (xx < nx && yy < ny) A.SP[0][fbase + ((long long)xx * nz + z) * ny + yy] = tile[tx][ty + k * kAliRows];
+    for (int k = 0; k < KR; ++k) {
+      const int xx = x0 + ty + k * ROWS, yy = y0 + tx;
+      if (xx < nx && yy < ny) A.SP[0][fbase + ((long long)xx * nz + z) * ny + yy] = tile[tx][ty + k * ROWS];
     }
   }
   block_max_to(fmax(rmax, (double)rmaxf), &A.st->resid_bits);
@@ -2189,7 +2208,10 @@ template <typename T>
 cudaError_t launch_ali(const AliArgs<T> &A, cudaStream_t s) {
   const dim3 grid((unsigned)(((A.d.n[0] + kAliTile - 1) / kAliTile) * ((A.d.n[1] + kAliTile - 1) / kAliTile)),
                   (unsigned)A.d.n[2], (unsigned)A.d.nf);
-  ali_update_kernel<T><<<grid, kAliTile * kAliRows, 0, s>>>(A);
+  if ((long long)grid.x * grid.y * grid.z <= kAliWideBlocks)
+    ali_update_kernel<T, kAliTile><<<grid, kAliTile * kAliTile, 0, s>>>(A);
+  else
+    ali_update_kernel<T, kAliRows><<<grid, kAliTile * kAliRows, 0, s>>>(A);
   return cudaGetLastError();
 }
 
