@@ -1674,38 +1674,50 @@ __global__ void state_op_kernel(SolveState *st, int op, int a, double b, int c) 
 // ------------------------------------------------------------------- Lambda*
 // Lambda*_ii = sum_k w_k Psi0_k(i) and 1 - Lambda*_ii = sum_k w_k (1 - Psi0_k(i)),
 // from chi alone, with the sweep's precision T for the segment weights; the sums
-// are FP64 (float32 grids: exact float pairs).  The rays' constants are staged in
-// shared memory; each thread owns one cell and frequency.
+// are FP64 (float32 grids: exact float pairs).  A block owns 32 x 16 cells (x, y) of
+// one z plane and frequency, two a thread: chi of its three planes is converted and
+// its boundaries resolved once, in shared memory, and a ray is four offsets there
+// (converting and locating four FP64 neighbours a ray and cell took most of the
+// time: the FP64 pipe converts 2 a clock and SM; 15 ms at 256^3 x 48 rays).  With the
+// FP64 weights and the block-wise smallest epsilon, set-up there is 33 ms shorter.
 template <typename T>
-struct LstarRay {
+struct __align__(16) LstarRay {
   T w4[4];            // weights of the four upwind face vertices
+  int off[4];         // the four vertices, as offsets in the tile
   T hs;               // half the path length, s/2
-  double w;           // quadrature weight
-  signed char off[4][3];   // canonical offsets (x, y, z) of the four vertices
+  T w;                // quadrature weight
+  T pad[2];
 };
 constexpr int kLstarChunk = 64;   // rays staged in shared memory at a time
+constexpr int kLstarX = 32, kLstarY = 16, kLstarW = kLstarX + 2, kLstarP = kLstarW * (kLstarY + 2);
 
 template <typename T>
 __global__ void __launch_bounds__(256) lstar_kernel(Dims d, const double *chi, const RayGeom *rays,
                                                     int na, double *lstar, double *oml,
                                                     const double *xchi_lo, const double *xchi_hi) {
   __shared__ LstarRay<T> R[kLstarChunk];
-  const long long cells = d.cells;
-  const long long N = cells * d.nf;
+  __shared__ T tile[3 * kLstarP];
   const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
   const int px = d.periodic[0], py = d.periodic[1], pz = d.periodic[2];
-  // every block walks the same cell range in the same chunks, so the barriers match
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long nloop = (N + stride - 1) / stride;
-  for (long long it = 0; it < nloop; ++it) {
-    const long long i = it * stride + blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const bool live = i < N;
-    const long long f = live ? i / cells : 0, c = live ? i - f * cells : 0;
-    const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-    const double *chf = chi + f * cells;
-    const T chi0 = live ? (T)chf[c] : T(0);
-    // float32 sums kept exact as a float pair (TwoSum); FP64 sums directly
-    T Lh = T(0), Ll = T(0), Oh = T(0), Ol = T(0);
+  const int tiles_x = (nx + kLstarX - 1) / kLstarX;
+  const int x0 = (int)(blockIdx.x % tiles_x) * kLstarX, y0 = (int)(blockIdx.x / tiles_x) * kLstarY;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (long long zf = blockIdx.y; zf < (long long)nz * d.nf; zf += gridDim.y) {
+    const int f = (int)(zf / nz), z = (int)(zf - (long long)f * nz);
+    const double *chf = chi + f * d.cells;
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * kLstarP; i += 256) {
+      const int k = i / kLstarP, r = (i - k * kLstarP) / kLstarW;
+      int xx = x0 - 1 + i - k * kLstarP - r * kLstarW, yy = y0 - 1 + r, zz = z - 1 + k;
+      xx = xx < 0 ? (px ? nx - 1 : 0) : (xx >= nx ? (px && xx == nx ? 0 : nx - 1) : xx);
+      yy = yy < 0 ? (py ? ny - 1 : 0) : (yy >= ny ? (py && yy == ny ? 0 : ny - 1) : yy);
+      // beyond a subdomain z face: the ghost layer's chi
+      const double *xc = zz < 0 ? xchi_lo : (zz >= nz ? xchi_hi : nullptr);
+      zz = zz < 0 ? (pz ? nz - 1 : 0) : (zz >= nz ? (pz ? 0 : nz - 1) : zz);
+      tile[i] = (T)(xc ? xc[((long long)f * ny + yy) * nx + xx] : chf[((long long)zz * ny + yy) * nx + xx]);
+    }
+    const T *own = tile + kLstarP + (ty + 1) * kLstarW + tx + 1;
+    PartSum<T> L[2], O[2];
     for (int k0 = 0; k0 < na; k0 += kLstarChunk) {
       const int nk = min(kLstarChunk, na - k0);
       __syncthreads();
@@ -1713,57 +1725,44 @@ __global__ void __launch_bounds__(256) lstar_kernel(Dims d, const double *chi, c
         const RayGeom r = rays[k0 + threadIdx.x];
         LstarRay<T> q;
         const int ax = r.axis, b1 = (ax + 1) % 3, b2 = (ax + 2) % 3;
-        const double f1 = b1 == 0 ? r.frac[0] : (b1 == 1 ? r.frac[1] : r.frac[2]);
-        const double f2 = b2 == 0 ? r.frac[0] : (b2 == 1 ? r.frac[1] : r.frac[2]);
+        const int step[3] = {1, kLstarW, kLstarP};
+        const int s0 = -r.sgn[ax] * step[ax], s1 = -r.sgn[b1] * step[b1], s2 = -r.sgn[b2] * step[b2];
+        const double f1 = r.frac[b1], f2 = r.frac[b2];
         for (int v = 0; v < 4; ++v) {
           const int d1 = v >> 1, d2 = v & 1;
           q.w4[v] = (T)((d1 ? f1 : 1.0 - f1) * (d2 ? f2 : 1.0 - f2));
-          int o[3] = {0, 0, 0};
-          o[ax] = -r.sgn[ax];
-          o[b1] = -d1 * r.sgn[b1];
-          o[b2] = -d2 * r.sgn[b2];
-          for (int a = 0; a < 3; ++a) q.off[v][a] = (signed char)o[a];
+          q.off[v] = s0 + d1 * s1 + d2 * s2;
         }
         q.hs = (T)(0.5 * r.s);
-        q.w = r.w;
+        q.w = (T)r.w;
+        q.pad[0] = q.pad[1] = T(0);
         R[threadIdx.x] = q;
       }
       __syncthreads();
-      if (!live) continue;
       for (int k = 0; k < nk; ++k) {
         const LstarRay<T> &q = R[k];
-        T chim = T(0);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          int xx = x + q.off[v][0], yy = y + q.off[v][1], zz = z + q.off[v][2];
-          xx = xx < 0 ? (px ? nx - 1 : 0) : (xx >= nx ? (px ? 0 : nx - 1) : xx);
-          yy = yy < 0 ? (py ? ny - 1 : 0) : (yy >= ny ? (py ? 0 : ny - 1) : yy);
-          // beyond a subdomain z face: the ghost layer's chi
-          const double *xc = zz < 0 ? xchi_lo : (zz >= nz ? xchi_hi : nullptr);
-          zz = zz < 0 ? (pz ? nz - 1 : 0) : (zz >= nz ? (pz ? 0 : nz - 1) : zz);
-          chim += q.w4[v] * (T)(xc ? xc[(f * ny + yy) * nx + xx] : chf[((long long)zz * ny + yy) * nx + xx]);
-        }
-        const T dtau = (chim + chi0) * q.hs;
-        T E, psi0, om;
-        seg_weights(dtau, E, psi0, om);
-        const T wl = (T)q.w * psi0, wo = (T)q.w * om;
-        if (sizeof(T) == 4) {
-          T s2 = Lh + wl, bp = s2 - Lh;
-          Ll += (Lh - (s2 - bp)) + (wl - bp);
-          Lh = s2;
-          s2 = Oh + wo;
-          bp = s2 - Oh;
-          Ol += (Oh - (s2 - bp)) + (wo - bp);
-          Oh = s2;
-        } else {
-          Lh += q.w * (double)psi0;
-          Oh += q.w * (double)om;
+        for (int c = 0; c < 2; ++c) {
+          const T *at = own + c * (kLstarY / 2) * kLstarW;
+          T chim = T(0);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) chim += q.w4[v] * at[q.off[v]];
+          const T dtau = (chim + at[0]) * q.hs;
+          T E, psi0, om;
+          seg_weights(dtau, E, psi0, om);
+          L[c].add(q.w * psi0);
+          O[c].add(q.w * om);
         }
       }
     }
-    if (live) {
-      lstar[i] = (double)Lh + (double)Ll;
-      oml[i] = (double)Oh + (double)Ol;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int x = x0 + tx, y = y0 + ty + c * (kLstarY / 2);
+      if (x < nx && y < ny) {
+        const long long i = f * d.cells + ((long long)z * ny + y) * nx + x;
+        lstar[i] = L[c].total();
+        oml[i] = O[c].total();
+      }
     }
   }
 }
@@ -1939,12 +1938,25 @@ __global__ void __launch_bounds__(kAliTile * kAliRows, 4) reduce_moments_kernel(
   }
 }
 
-__global__ void eps_thick_min_kernel(Dims d, const double *eps, const double *oml,
-                                     unsigned long long *out) {
-  const long long N = d.cells * d.nf;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    if (oml[i] < 0.5) atomicMin(&out[i / d.cells], (unsigned long long)__double_as_longlong(eps[i]));
+// One frequency per blockIdx.y, one atomic a block (one a cell, all of a frequency's
+// on the same word, took 2.5 ms at 256^3).
+__global__ void __launch_bounds__(256) eps_thick_min_kernel(Dims d, const double *eps, const double *oml,
+                                                            unsigned long long *out) {
+  __shared__ unsigned long long red[8];
+  for (int f = blockIdx.y; f < d.nf; f += gridDim.y) {
+    unsigned long long m = ~0ULL;   // (eps > 0: the bits order as the values do)
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < d.cells;
+         i += (long long)gridDim.x * blockDim.x)
+      if (oml[f * d.cells + i] < 0.5)
+        m = min(m, (unsigned long long)__double_as_longlong(eps[f * d.cells + i]));
+    for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) m = min(m, red[w]);
+      if (m != ~0ULL) atomicMin(&out[f], m);
+    }
+    __syncthreads();
   }
 }
 
@@ -2239,9 +2251,10 @@ cudaError_t launch_state_op(SolveState *st, int op, int a, double b, int c, cuda
 template <typename T>
 cudaError_t launch_lstar(const Dims &d, const double *chi, const RayGeom *rays, int na, double *lstar,
                          double *oml, const double *const xchi[2], cudaStream_t s) {
-  lstar_kernel<T><<<grid_for(d.cells * d.nf, 256), 256, 0, s>>>(d, chi, rays, na, lstar, oml,
-                                                                 xchi ? xchi[0] : nullptr,
-                                                                 xchi ? xchi[1] : nullptr);
+  const dim3 grid((unsigned)(((d.n[0] + kLstarX - 1) / kLstarX) * ((d.n[1] + kLstarY - 1) / kLstarY)),
+                  (unsigned)std::min<long long>((long long)d.n[2] * d.nf, 65535), 1);
+  lstar_kernel<T><<<grid, 256, 0, s>>>(d, chi, rays, na, lstar, oml, xchi ? xchi[0] : nullptr,
+                                       xchi ? xchi[1] : nullptr);
   return cudaGetLastError();
 }
 
@@ -2298,7 +2311,9 @@ cudaError_t launch_inv_denominator(long long n, const double *eps, const double 
 
 cudaError_t launch_eps_thick_min(const Dims &d, const double *eps, const double *oml,
                                  unsigned long long *out, cudaStream_t s) {
-  eps_thick_min_kernel<<<grid_for(d.cells * d.nf, 256), 256, 0, s>>>(d, eps, oml, out);
+  const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>((d.cells + 2047) / 2048, 608)),
+                  (unsigned)std::min(d.nf, 65535));
+  eps_thick_min_kernel<<<grid, 256, 0, s>>>(d, eps, oml, out);
   return cudaGetLastError();
 }
 
