@@ -357,12 +357,27 @@ rt_status rt_get_stats(rt_grid g, rt_stats *out);
  * runtime's count of co-resident clusters and a cost model (rt_autotune measures
  * instead).  Variant 3, and FP64's automatic choice, take the segment weights
  * from a table of two values per ray and cell, filled once per medium and plan
- * and kept by the grid, where that takes at most a quarter of the free device
- * memory, and form them as they sweep otherwise.
+ * and kept by the grid (the streamed sweep), where that takes at most a quarter of
+ * the free device memory (rt_set_table_limit), and form them as they sweep
+ * otherwise.
  * Results do not depend on the configuration beyond rounding order.
  * Errors: RT_ERR_ARG for out-of-range values or no feasible configuration. */
 rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas, int threads,
                               int variant);
+
+/* Largest table of segment weights the grid may hold, in bytes (see
+ * rt_set_sweep_config): 0 for none, -1 (the default) for the automatic rule.
+ * Checked when the next solve would fill the table: where it is larger, the grid
+ * is planned without it (variant 3 then is the pipelined sweep).  Also applies to
+ * a mixed grid's internal FP64 grids.  Frees a table that is too large now and
+ * replans the sweep.  Errors: RT_ERR_ARG for bytes < -1. */
+rt_status rt_set_table_limit(rt_grid g, long long bytes);
+
+/* Whether the sweep as planned reads its weights from the table (*streams 1 or 0;
+ * before the first solve of a medium: whether it will if there is room), and the
+ * bytes of the tables the grid and its internal FP64 grids hold.  Either pointer
+ * may be NULL. */
+rt_status rt_get_sweep_table(rt_grid g, int *streams, long long *bytes);
 
 /* The sweep plan in use (7 ints): plan[0] variant, [1] groups per frequency,
  * [2] rays per group (max), [3] strips per plane (cluster size), [4] threads per

@@ -376,7 +376,9 @@ struct rt_grid_s {
   void *wt = nullptr;
   size_t wt_bytes = 0;
   long long wt_gen = -1;
-  bool wt_off = false;                // the table did not fit in device memory
+  long long wt_limit = -1;            // largest table (rt_set_table_limit; < 0: automatic)
+  bool wt_never = false;              // no table whatever the room (subdomain faces, no allocations)
+  bool wt_off = false;                // the table did not fit
   long long graph_launches = 0;
 };
 
@@ -676,7 +678,7 @@ int stream_resident(rt_grid g, const StreamShape &sh, int C) {
 // configuration fits.
 bool plan_stream(rt_grid g) {
   const bool f64 = g->desc.prec == RT_PREC_FP64;
-  if (g->interp != RT_INTERP_LINEAR || g->wt_off || external_faces(g)) return false;
+  if (g->interp != RT_INTERP_LINEAR || g->wt_never || g->wt_off || external_faces(g)) return false;
   if (!(g->req_variant == 3 || g->req_variant == 0)) return false;
   int minNv = 1 << 30;
   for (int a = 0; a < 3; ++a) {
@@ -1002,12 +1004,12 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
 
 // The segment weights E, Psi0 are functions of chi alone: the streamed sweep, and
 // the one-cell-per-thread sweep of FP64 grids, read them from a table filled once
-// per medium and plan.  A table takes at most a quarter of the free device memory;
-// without the room the grid is planned without it (the sweeps then compute the
+// per medium and plan.  A table takes at most a quarter of the free device memory
+// (or what rt_set_table_limit allows); without the room the grid is planned without it (the sweeps then compute the
 // weights as they go).
 template <typename T>
 rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
-  if (g->wt_off || !(g->stream || (sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR))) return RT_OK;
+  if (g->wt_never || g->wt_off || !(g->stream || (sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR))) return RT_OK;
   if (g->wt && g->wt_gen == g->gen) return RT_OK;
   const size_t slots = g->group_angles.size();
   const size_t need = g->stream ? slots * g->d.nf * rtk::stream_slot_elems<T>(g->d, g->used_axis) * sizeof(T)
@@ -1017,7 +1019,8 @@ rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
     g->wt = nullptr;
     g->wt_bytes = 0;
     size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || (g->stream && need > fr / 4) ||
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess ||
+        (g->wt_limit >= 0 ? need > (size_t)g->wt_limit : g->stream && need > fr / 4) ||
         cudaMalloc(&g->wt, need) != cudaSuccess) {
       cudaGetLastError();
       g->wt = nullptr;
@@ -1608,6 +1611,7 @@ rt_status plan_bins(rt_grid g) {
     if (r != RT_OK) return r;
     if ((r = rt_set_interpolation(g->sub64, g->interp)) != RT_OK) return r;
     if ((r = rt_set_iteration(g->sub64, g->iteration)) != RT_OK) return r;
+    g->sub64->wt_limit = g->wt_limit;
     g->bins64 = ill;
   }
   const size_t C = (size_t)g->d.cells, m = ill.size();
@@ -1648,10 +1652,11 @@ rt_status plan_first64(rt_grid g) {
     rt_status r = rt_create_grid(&d, &g->first64);
     if (r != RT_OK) return r;
     g->first64->shadow = true;
+    g->first64->wt_limit = g->wt_limit;
     // a few FP64 iterations per solve: their segment weights are tabulated per
     // medium when the table is modest (it holds E and Psi0 of every ray and cell)
     if (2.0 * g->na * (double)N_of(g) * 8.0 > kShadowTableMax) {
-      g->first64->wt_off = true;
+      g->first64->wt_never = true;
       plan_groups(g->first64);
       if ((r = upload_plan_any(g->first64)) != RT_OK) return r;
     }
@@ -1791,7 +1796,7 @@ rt_status rt_create_grid(const rt_grid_desc *desc, rt_grid *out) {
         cudaMemset(g->xB[side], 0, lay) != cudaSuccess || cudaMemset(g->xI[side], 0, ray) != cudaSuccess ||
         cudaMemset(g->xout[side], 0, ray) != cudaSuccess)
       return cleanup(fail(RT_ERR_CUDA, "initialisation of the subdomain face buffers failed"));
-    g->wt_off = true;   // the segment-weight table does not see the ghost layer's chi
+    g->wt_never = true;   // the segment-weight table does not see the ghost layer's chi
   }
   ALLOC(g->rays_d, (size_t)g->na * sizeof(RayGeom));
   ALLOC(g->st, sizeof(rtk::SolveState));
@@ -1902,6 +1907,35 @@ rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas,
   if (g->groups.empty()) return fail(RT_ERR_ARG, "no feasible sweep configuration");
   if (g->smem > 227 * 1024) return fail(RT_ERR_ARG, "sweep configuration needs %zu bytes of shared memory", g->smem);
   return upload_plan_any(g);
+}
+
+rt_status rt_set_table_limit(rt_grid g, long long bytes) {
+  if (!g) return fail(RT_ERR_ARG, "NULL grid");
+  if (bytes < -1) return fail(RT_ERR_ARG, "the table limit must be >= 0, or -1 for automatic");
+  cudaStreamSynchronize(g->own);
+  g->wt_limit = bytes;
+  if (g->wt && bytes >= 0 && g->wt_bytes > (size_t)bytes) {
+    cudaFree(g->wt);   // (waits for the sweeps that read it)
+    g->wt = nullptr;
+    g->wt_bytes = 0;
+  }
+  g->wt_off = false;   // decided again at the next solve
+  plan_groups(g);
+  rt_status r = upload_plan_any(g);
+  for (rt_grid h : {g->first64, g->sub64})
+    if (r == RT_OK && h) r = rt_set_table_limit(h, bytes);
+  return r;
+}
+
+rt_status rt_get_sweep_table(rt_grid g, int *streams, long long *bytes) {
+  if (!g) return fail(RT_ERR_ARG, "NULL grid");
+  if (streams) *streams = g->stream ? 1 : 0;
+  if (bytes) {
+    *bytes = (long long)g->wt_bytes;
+    for (rt_grid h : {g->first64, g->sub64})
+      if (h) *bytes += (long long)h->wt_bytes;
+  }
+  return RT_OK;
 }
 
 rt_status rt_set_opacity_source(rt_grid g, const double *chi_tot, const double *eps, const double *B,
@@ -2917,7 +2951,7 @@ extern "C" rt_status rt_formal_solve_noalloc(const rt_grid_desc *desc, const dou
   }
   // the size limit is checked before any pointer is touched
   rt_grid_s g;
-  g.wt_off = true;   // no segment-weight table: this entry point allocates nothing
+  g.wt_never = true;   // no segment-weight table: this entry point allocates nothing
   g.desc = D;
   g.two_d = D.nz == 1;
   if (g.two_d) {

@@ -97,6 +97,8 @@ _SIGS = {
     "rt_get_stats": (ctypes.c_int, [_VP, ctypes.POINTER(rt_stats)]),
     "rt_set_sweep_config": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "rt_get_sweep_plan": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_int)]),
+    "rt_set_table_limit": (ctypes.c_int, [_VP, ctypes.c_longlong]),
+    "rt_get_sweep_table": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_longlong)]),
     "rt_autotune": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_int)]),
     "rt_angle_table": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, _VP, _VP]),
     "rt_formal_solve_noalloc": (ctypes.c_int, [ctypes.POINTER(rt_grid_desc), _VP, _VP, _VP, _VP, _VP]),
@@ -300,6 +302,16 @@ class Grid:
         _check(load().rt_get_sweep_plan(self._h, v))
         return dict(zip(("variant", "groups", "rays_per_group", "cluster", "threads", "smem", "fp64_bins"),
                         list(v)))
+
+    def set_table_limit(self, nbytes=-1):
+        """Largest table of segment weights, 0 for none, -1 for automatic (rt_set_table_limit)."""
+        _check(load().rt_set_table_limit(self._h, int(nbytes)))
+
+    def sweep_table(self):
+        """Whether the sweep streams its weights from a table, and the tables' bytes (rt_get_sweep_table)."""
+        streams, n = ctypes.c_int(0), ctypes.c_longlong(0)
+        _check(load().rt_get_sweep_table(self._h, ctypes.byref(streams), ctypes.byref(n)))
+        return {"streams": bool(streams.value), "bytes": n.value}
 
     def set_opacity_source(self, chi, eps, B, freq_w=None):
         pc, dc, kc = self._in(chi)
