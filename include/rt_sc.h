@@ -360,8 +360,11 @@ rt_status rt_get_stats(rt_grid g, rt_stats *out);
  * and kept by the grid (the streamed sweep), where that takes at most a quarter of
  * the free device memory (rt_set_table_limit), and form them as they sweep
  * otherwise.
- * Results do not depend on the configuration beyond rounding order.
- * Errors: RT_ERR_ARG for out-of-range values or no feasible configuration. */
+ * Results do not depend on the configuration beyond rounding order.  Rays and strips
+ * that fit the streamed sweep alone are set aside where the grid has to sweep without
+ * the table.
+ * Errors: RT_ERR_ARG for out-of-range values or no feasible configuration (the plan
+ * then stays as it was). */
 rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas, int threads,
                               int variant);
 

@@ -464,6 +464,7 @@ void build_rays(rt_grid g) {
 // Largest dynamic shared memory a sweep CTA may use.
 constexpr size_t kSweepSmemBudget = 200 * 1024;
 constexpr size_t kStreamSmemBudget = 224 * 1024;
+constexpr size_t kSmemMax = 227 * 1024;   // of a CTA on this GPU: a launch that asks for more fails
 constexpr int kSMs = 152;
 
 int amax_for(int apg) { return apg <= 1 ? 1 : (apg <= 2 ? 2 : (apg <= 4 ? 4 : 8)); }
@@ -748,7 +749,10 @@ bool plan_stream(rt_grid g) {
 // (waves of resident clusters) x (rays per group) x (cells per strip) x
 // (CTAs sharing an SM), from the runtime's count of co-resident clusters
 // (clusters cannot straddle a GPC, so this is not simply SMs / C).
-void plan_groups(rt_grid g) {
+// A request that the grid's present kernel has no shared memory for (it was made for
+// the streamed sweep, or for linear interpolation) is dropped from this plan, but kept
+// for later ones; with `strict` the plan is left too large, which its caller refuses.
+void plan_groups(rt_grid g, bool strict = false) {
   g->stream = false;
   if (plan_stream(g)) return;
   int minNv = 1 << 30;
@@ -824,6 +828,15 @@ void plan_groups(rt_grid g) {
   g->cluster = bC;
   sweep_shape(g, variant, namax, bC, &g->smem, &g->threads);
   if (g->req_threads > 0) g->threads = std::min(g->req_threads, sweep_thread_cap(g, variant));
+  if (g->smem > kSmemMax && !strict && (g->req_apg || g->req_cluster || g->req_threads)) {
+    const int req[3] = {g->req_apg, g->req_cluster, g->req_threads};
+    g->req_apg = g->req_cluster = g->req_threads = 0;
+    plan_groups(g);
+    g->req_apg = req[0];
+    g->req_cluster = req[1];
+    g->req_threads = req[2];
+    return;
+  }
   split_last_wave(g);
 }
 
@@ -1899,13 +1912,25 @@ rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas,
   if ((g->xI[0] || g->xI[1]) && variant > 1)
     return fail(RT_ERR_ARG, "a grid with subdomain z faces sweeps one cell per thread (variant 1)");
   cudaStreamSynchronize(g->own);
+  const int before[4] = {g->req_apg, g->req_cluster, g->req_threads, g->req_variant};
   g->req_apg = angles_per_group;
   g->req_cluster = cluster_ctas;
   g->req_threads = threads;
   g->req_variant = variant;
-  plan_groups(g);
-  if (g->groups.empty()) return fail(RT_ERR_ARG, "no feasible sweep configuration");
-  if (g->smem > 227 * 1024) return fail(RT_ERR_ARG, "sweep configuration needs %zu bytes of shared memory", g->smem);
+  plan_groups(g, true);
+  const bool none = g->groups.empty();
+  const size_t smem = g->smem;
+  if (none || smem > kSmemMax) {   // refused: the plan stays as it was
+    g->req_apg = before[0];
+    g->req_cluster = before[1];
+    g->req_threads = before[2];
+    g->req_variant = before[3];
+    plan_groups(g);
+    rt_status r = upload_plan_any(g);
+    if (r != RT_OK) return r;
+    return none ? fail(RT_ERR_ARG, "no feasible sweep configuration")
+                : fail(RT_ERR_ARG, "sweep configuration needs %zu bytes of shared memory", smem);
+  }
   return upload_plan_any(g);
 }
 

@@ -81,6 +81,30 @@ def test_formal_solutions_iterations_and_moments(rt, case):
         assert t["streams"] and t["bytes"] > 0
 
 
+@pytest.mark.parametrize("prec,shape,cfg", [("mixed", (256, 256, 16), dict(angles_per_group=3, cluster_ctas=16)),
+                                            ("fp64", (128, 128, 16), dict(angles_per_group=2, cluster_ctas=6))])
+def test_a_plan_that_only_the_streamed_sweep_fits(rt, prec, shape, cfg):
+    """Such rays and strips (the pipelined sweep would need 238 and 268 KB of shared
+    memory a CTA for them) are set aside when the table has no room, and taken again
+    when it has; asked for without the room they are an error that leaves the grid
+    as it was."""
+    p = W.random_box(*shape, seed=430, n_mu=6, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    ref = O.formal_solution(O.Grid.from_problem(p), p.chi[0], p.B[0], p.B[0], nthreads=O.max_threads())["J"]
+    tol = 1e-10 if prec == "fp64" else 1e-5
+    with _grid(rt, p, prec, dict(cfg, variant=3)) as g:
+        plan = lambda: (g.sweep_plan()["rays_per_group"], g.sweep_plan()["cluster"])
+        assert plan() == tuple(cfg.values())
+        assert rel(g.formal_solve(p.B)[0], ref) < tol
+        assert not g.sweep_table()["streams"] and plan() != tuple(cfg.values())
+        with pytest.raises(rt.RTError) as e:
+            g.set_sweep_config(**cfg, variant=3)
+        assert e.value.status == rt.RT_ERR_ARG
+        assert rel(g.formal_solve(p.B)[0], ref) < tol
+        g.set_table_limit(-1)
+        assert rel(g.formal_solve(p.B)[0], ref) < tol
+        assert g.sweep_table()["streams"] and plan() == tuple(cfg.values())
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_gauss_seidel(rt, prec):
     """One iteration (the forward phase by the sweep, S by the reverse phase)."""
