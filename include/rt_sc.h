@@ -391,7 +391,8 @@ rt_status rt_get_sweep_plan(rt_grid g, int *plan);
 /* Time candidate sweep configurations (variant x rays per group x strips) with
  * formal solutions of the current medium, keep the fastest for this grid and
  * remember it for every later grid of the same shape, rays, frequencies,
- * precision and boundaries in this process.  Leaves S = B and fresh ghosts (as
+ * precision and boundaries in this process (grids with and without room for the
+ * table of segment weights apart).  Leaves S = B and fresh ghosts (as
  * rt_set_opacity_source does).  plan_out (7 ints, may be NULL) receives the plan
  * as rt_get_sweep_plan reports it.  Errors: RT_ERR_STATE before
  * rt_set_opacity_source. */

@@ -1020,21 +1020,33 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
 // per medium and plan.  A table takes at most a quarter of the free device memory
 // (or what rt_set_table_limit allows); without the room the grid is planned without it (the sweeps then compute the
 // weights as they go).
+size_t stream_table_bytes(rt_grid g) {
+  return (size_t)g->na * g->d.nf * g->tsize *
+         (g->desc.prec == RT_PREC_FP64 ? rtk::stream_slot_elems<double>(g->d, g->used_axis)
+                                       : rtk::stream_slot_elems<float>(g->d, g->used_axis));
+}
+// whether a table of `need` bytes may be allocated now (one that the grid holds would be freed first)
+bool table_room(rt_grid g, size_t need, bool stream) {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return g->wt_limit >= 0 ? need <= (size_t)g->wt_limit : !stream || need <= (fr + g->wt_bytes) / 4;
+}
+
 template <typename T>
 rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
   if (g->wt_never || g->wt_off || !(g->stream || (sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR))) return RT_OK;
   if (g->wt && g->wt_gen == g->gen) return RT_OK;
   const size_t slots = g->group_angles.size();
-  const size_t need = g->stream ? slots * g->d.nf * rtk::stream_slot_elems<T>(g->d, g->used_axis) * sizeof(T)
-                                : 2 * slots * (size_t)N_of(g) * sizeof(T);
+  const size_t need = g->stream ? stream_table_bytes(g) : 2 * slots * (size_t)N_of(g) * sizeof(T);
   if (need > g->wt_bytes) {
+    const bool room = table_room(g, need, g->stream);
     if (g->wt) cudaFree(g->wt);
     g->wt = nullptr;
     g->wt_bytes = 0;
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess ||
-        (g->wt_limit >= 0 ? need > (size_t)g->wt_limit : g->stream && need > fr / 4) ||
-        cudaMalloc(&g->wt, need) != cudaSuccess) {
+    if (!room || cudaMalloc(&g->wt, need) != cudaSuccess) {
       cudaGetLastError();
       g->wt = nullptr;
       g->wt_off = true;
@@ -2389,9 +2401,11 @@ rt_status rt_enable_timing(rt_grid g, int enable) {
   return RT_OK;
 }
 
-// Plans chosen by rt_autotune, keyed by problem shape (process-wide cache).
+// Plans chosen by rt_autotune, keyed by problem shape and by whether the table of
+// segment weights has room: the kernels that were timed are others without it
+// (process-wide cache).
 struct TuneKey {
-  int n[3], nf, n_mu, prec, bc[6], interp, iteration;
+  int n[3], nf, n_mu, prec, bc[6], interp, iteration, table;
   bool operator==(const TuneKey &o) const { return std::memcmp(this, &o, sizeof(TuneKey)) == 0; }
 };
 struct TuneVal {
@@ -2413,6 +2427,8 @@ TuneKey tune_key(rt_grid g) {
   k.prec = g->desc.prec;
   k.interp = g->interp;
   k.iteration = g->iteration;
+  const size_t need = stream_table_bytes(g);
+  k.table = g->interp != RT_INTERP_LINEAR || (!g->wt_never && !g->wt_off && (g->wt_bytes >= need || table_room(g, need, true)));
   return k;
 }
 
@@ -2420,6 +2436,7 @@ rt_status rt_autotune(rt_grid g, int *plan_out) {
   if (!g) return fail(RT_ERR_ARG, "NULL grid");
   if (!g->have_medium) return fail(RT_ERR_STATE, "rt_set_opacity_source has not succeeded");
   const TuneKey key = tune_key(g);
+  if (!key.table) g->wt_off = true;        // (until a medium or a limit that makes room)
   TuneVal best{0, 0, 0, 0};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);

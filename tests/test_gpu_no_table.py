@@ -105,6 +105,22 @@ def test_a_plan_that_only_the_streamed_sweep_fits(rt, prec, shape, cfg):
         assert g.sweep_table()["streams"] and plan() == tuple(cfg.values())
 
 
+@pytest.mark.parametrize("first", [None, 0])
+def test_tuned_plans_are_not_shared_with_grids_that_have_a_table(rt, first):
+    """The cache answers a second grid of the same kind, and no grid of the other."""
+    p = W.random_box(24, 20, 16 if first is None else 18, seed=440, n_mu=2)
+    tuned = {}
+    for limit in (first, -1 if first == 0 else 0):
+        for again in range(2):
+            with _grid(rt, p, "mixed", {}, limit) as g:
+                plan, n = g.autotune(), g.stats()["kernel_launches"]
+                J = g.formal_solve(p.B)
+                assert limit != 0 or not g.sweep_table()["streams"]
+                assert (n < 50) == bool(again), n        # a search launches hundreds of kernels
+                assert tuned.setdefault(limit, plan) == plan
+                np.testing.assert_allclose(J, tuned.setdefault("J", J), rtol=1e-5)
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_gauss_seidel(rt, prec):
     """One iteration (the forward phase by the sweep, S by the reverse phase)."""
