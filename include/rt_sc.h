@@ -358,8 +358,8 @@ rt_status rt_get_stats(rt_grid g, rt_stats *out);
  * instead).  Variant 3, and FP64's automatic choice, take the segment weights
  * from a table of two values per ray and cell, filled once per medium and plan
  * and kept by the grid (the streamed sweep), where that takes at most a quarter of
- * the free device memory (rt_set_table_limit), and form them as they sweep
- * otherwise.
+ * the free device memory (FP64's automatic choice: what there is; rt_set_table_limit
+ * for another limit), and form them as they sweep otherwise.
  * Results do not depend on the configuration beyond rounding order.  Rays and strips
  * that fit the streamed sweep alone are set aside where the grid has to sweep without
  * the table.

@@ -378,7 +378,8 @@ struct rt_grid_s {
   long long wt_gen = -1;
   long long wt_limit = -1;            // largest table (rt_set_table_limit; < 0: automatic)
   bool wt_never = false;              // no table whatever the room (subdomain faces, no allocations)
-  bool wt_off = false;                // the table did not fit
+  bool no_stream = false;             // the streamed sweep's table did not fit
+  bool wt_off = false;                // ... nor the one-cell-per-thread sweep's
   long long graph_launches = 0;
 };
 
@@ -679,7 +680,7 @@ int stream_resident(rt_grid g, const StreamShape &sh, int C) {
 // configuration fits.
 bool plan_stream(rt_grid g) {
   const bool f64 = g->desc.prec == RT_PREC_FP64;
-  if (g->interp != RT_INTERP_LINEAR || g->wt_never || g->wt_off || external_faces(g)) return false;
+  if (g->interp != RT_INTERP_LINEAR || g->wt_never || g->no_stream || external_faces(g)) return false;
   if (!(g->req_variant == 3 || g->req_variant == 0)) return false;
   int minNv = 1 << 30;
   for (int a = 0; a < 3; ++a) {
@@ -1018,41 +1019,52 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
 // The segment weights E, Psi0 are functions of chi alone: the streamed sweep, and
 // the one-cell-per-thread sweep of FP64 grids, read them from a table filled once
 // per medium and plan.  A table takes at most a quarter of the free device memory
-// (or what rt_set_table_limit allows); without the room the grid is planned without it (the sweeps then compute the
+// (FP64's automatic plan: all of it), or what rt_set_table_limit allows; without the
+// room the grid is planned without it (the sweeps then compute the
 // weights as they go).
 size_t stream_table_bytes(rt_grid g) {
   return (size_t)g->na * g->d.nf * g->tsize *
          (g->desc.prec == RT_PREC_FP64 ? rtk::stream_slot_elems<double>(g->d, g->used_axis)
                                        : rtk::stream_slot_elems<float>(g->d, g->used_axis));
 }
-// whether a table of `need` bytes may be allocated now (one that the grid holds would be freed first)
-bool table_room(rt_grid g, size_t need, bool stream) {
+// Whether a table of `need` bytes may be allocated now (one that the grid holds would
+// be freed first).  FP64 grids left to themselves take what there is: forming their
+// weights costs an exponential of the slow FP64 pipe an update (the one-cell-per-thread
+// sweep: 4.3 times the time).
+bool table_room(rt_grid g, size_t need) {
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return g->wt_limit >= 0 ? need <= (size_t)g->wt_limit : !stream || need <= (fr + g->wt_bytes) / 4;
+  if (g->wt_limit >= 0) return need <= (size_t)g->wt_limit;
+  const bool all = g->desc.prec == RT_PREC_FP64 && g->req_variant <= 1;
+  return need <= (all ? fr + g->wt_bytes : (fr + g->wt_bytes) / 4);
 }
 
 template <typename T>
 rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
-  if (g->wt_never || g->wt_off || !(g->stream || (sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR))) return RT_OK;
+  const bool one_cell = sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR && !g->wt_off;
+  if (g->wt_never || !(g->stream || one_cell)) return RT_OK;
   if (g->wt && g->wt_gen == g->gen) return RT_OK;
   const size_t slots = g->group_angles.size();
   const size_t need = g->stream ? stream_table_bytes(g) : 2 * slots * (size_t)N_of(g) * sizeof(T);
   if (need > g->wt_bytes) {
-    const bool room = table_room(g, need, g->stream);
+    const bool room = table_room(g, need);
     if (g->wt) cudaFree(g->wt);
     g->wt = nullptr;
     g->wt_bytes = 0;
     if (!room || cudaMalloc(&g->wt, need) != cudaSuccess) {
       cudaGetLastError();
       g->wt = nullptr;
-      g->wt_off = true;
-      if (!g->stream) return RT_OK;
+      if (!g->stream) {
+        g->wt_off = true;
+        return RT_OK;
+      }
+      g->no_stream = true;
       plan_groups(g);
-      return upload_plan<T>(g);
+      rt_status r = upload_plan<T>(g);
+      return r == RT_OK ? ensure_seg_table<T>(g, s) : r;   // (FP64: unpadded rows may fit)
     }
     g->wt_bytes = need;
     g->gen++;   // a new buffer: captured graphs must not replay the old pointers
@@ -1956,7 +1968,7 @@ rt_status rt_set_table_limit(rt_grid g, long long bytes) {
     g->wt = nullptr;
     g->wt_bytes = 0;
   }
-  g->wt_off = false;   // decided again at the next solve
+  g->no_stream = g->wt_off = false;   // decided again at the next solve
   plan_groups(g);
   rt_status r = upload_plan_any(g);
   for (rt_grid h : {g->first64, g->sub64})
@@ -2428,7 +2440,7 @@ TuneKey tune_key(rt_grid g) {
   k.interp = g->interp;
   k.iteration = g->iteration;
   const size_t need = stream_table_bytes(g);
-  k.table = g->interp != RT_INTERP_LINEAR || (!g->wt_never && !g->wt_off && (g->wt_bytes >= need || table_room(g, need, true)));
+  k.table = g->interp != RT_INTERP_LINEAR || (!g->wt_never && !g->no_stream && (g->wt_bytes >= need || table_room(g, need)));
   return k;
 }
 
@@ -2436,7 +2448,7 @@ rt_status rt_autotune(rt_grid g, int *plan_out) {
   if (!g) return fail(RT_ERR_ARG, "NULL grid");
   if (!g->have_medium) return fail(RT_ERR_STATE, "rt_set_opacity_source has not succeeded");
   const TuneKey key = tune_key(g);
-  if (!key.table) g->wt_off = true;        // (until a medium or a limit that makes room)
+  if (!key.table) g->no_stream = true;   // (until a medium or a limit that makes room)
   TuneVal best{0, 0, 0, 0};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);

@@ -3,6 +3,8 @@ grids take where the table has no room -- the float32 and FP64 pipelined sweeps,
 FP64 sweep of one cell per thread, their shared launches -- replanned at a grid's first
 solve.  Against the oracle; tolerances as in test_gpu_parity and test_gpu_stream
 (rounding only: 1e-10 FP64, 1e-5 float32)."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -36,6 +38,18 @@ def rt():
 def rel(a, b):
     a, b = np.asarray(a), np.asarray(b)
     return float(np.max(np.abs(a - b) / np.maximum(np.abs(b), 1e-300)))
+
+
+@contextlib.contextmanager
+def free_memory_of(nbytes):
+    """The device's free memory cut down to nbytes."""
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - nbytes, dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del hold
+        torch.cuda.empty_cache()
 
 
 def _grid(rt, p, prec, cfg, limit=0, scheme="jacobi"):
@@ -119,6 +133,28 @@ def test_tuned_plans_are_not_shared_with_grids_that_have_a_table(rt, first):
                 assert (n < 50) == bool(again), n        # a search launches hundreds of kernels
                 assert tuned.setdefault(limit, plan) == plan
                 np.testing.assert_allclose(J, tuned.setdefault("J", J), rtol=1e-5)
+
+
+def test_fp64_table_takes_the_memory_there_is(rt):
+    """A table of 0.68 GB in 1.2 GB of free memory."""
+    p = W.random_box(96, 96, 96, seed=450, n_mu=6)
+    with _grid(rt, p, "fp64", {}, None) as g:
+        with free_memory_of(1200 << 20):
+            J = g.formal_solve(p.B)
+            t = g.sweep_table()
+        assert t == {"streams": True, "bytes": 2 * 48 * 96 ** 3 * 8}
+        np.testing.assert_array_equal(J, g.formal_solve(p.B))
+
+
+def test_fp64_tables_of_unpadded_rows(rt):
+    """Rows of one cell: the streamed sweep's table (rows padded to 16 bytes) is twice
+    as large as the one-cell-per-thread sweep's, which fits the limit alone."""
+    p = W.random_box(1, 30, 20, seed=460, n_mu=4, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    ref = O.formal_solution(O.Grid.from_problem(p), p.chi[0], p.B[0], p.B[0])["J"]
+    small = 2 * 24 * 30 * 20 * 8
+    with _grid(rt, p, "fp64", {}, small) as g:
+        assert rel(g.formal_solve(p.B)[0], ref) < 1e-10
+        assert g.sweep_table() == {"streams": False, "bytes": small}
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
