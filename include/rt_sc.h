@@ -371,7 +371,8 @@ rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas,
 /* Largest table of segment weights the grid may hold, in bytes (see
  * rt_set_sweep_config): 0 for none, -1 (the default) for the automatic rule.
  * Checked when the next solve would fill the table: where it is larger, the grid
- * is planned without it (variant 3 then is the pipelined sweep).  Also applies to
+ * is planned without it (variant 3 then is the pipelined sweep), until a medium is
+ * set while there is room or the limit is set again.  Also applies to
  * a mixed grid's internal FP64 grids.  Frees a table that is too large now and
  * replans the sweep.  Errors: RT_ERR_ARG for bytes < -1. */
 rt_status rt_set_table_limit(rt_grid g, long long bytes);

@@ -378,7 +378,7 @@ struct rt_grid_s {
   long long wt_gen = -1;
   long long wt_limit = -1;            // largest table (rt_set_table_limit; < 0: automatic)
   bool wt_never = false;              // no table whatever the room (subdomain faces, no allocations)
-  bool no_stream = false;             // the streamed sweep's table did not fit
+  bool no_stream = false;             // the streamed sweep's table did not fit (until a medium that finds room)
   bool wt_off = false;                // ... nor the one-cell-per-thread sweep's
   long long graph_launches = 0;
 };
@@ -1993,6 +1993,11 @@ rt_status rt_set_opacity_source(rt_grid g, const double *chi_tot, const double *
   cudaStream_t s = g->own;
   const size_t N = (size_t)N_of(g);
   rt_status r;
+  if ((g->no_stream || g->wt_off) && table_room(g, stream_table_bytes(g))) {
+    g->no_stream = g->wt_off = false;   // a new medium, and now there is room for its table
+    plan_groups(g);
+    if ((r = upload_plan_any(g)) != RT_OK) return r;
+  }
   if ((r = copy_in(g, g->chi, chi_tot, N, on_device, s)) != RT_OK) return r;
   if ((r = copy_in(g, g->eps, eps, N, on_device, s)) != RT_OK) return r;
   if ((r = copy_in(g, g->B, B, N, on_device, s)) != RT_OK) return r;

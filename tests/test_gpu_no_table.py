@@ -146,6 +146,20 @@ def test_fp64_table_takes_the_memory_there_is(rt):
         np.testing.assert_array_equal(J, g.formal_solve(p.B))
 
 
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_a_later_medium_finds_the_room_that_an_earlier_one_had_not(rt, prec):
+    """A table of 0.27 GB (0.13 in float32) when 0.2 GB are free, and when all are."""
+    p = W.random_box(128, 128, 128, seed=470, n_mu=2)
+    with _grid(rt, p, prec, {}, None) as g:
+        with free_memory_of(200 << 20):
+            J = g.formal_solve(p.B)
+            assert g.sweep_table() == {"streams": False, "bytes": 0}
+        g.set_opacity_source(p.chi, p.eps, p.B, p.freq_w)
+        J2 = g.formal_solve(p.B)
+        assert g.sweep_table()["streams"]
+    np.testing.assert_allclose(J2, J, rtol=1e-12 if prec == "fp64" else 1e-5)
+
+
 def test_fp64_tables_of_unpadded_rows(rt):
     """Rows of one cell: the streamed sweep's table (rows padded to 16 bytes) is twice
     as large as the one-cell-per-thread sweep's, which fits the limit alone."""
