@@ -841,9 +841,16 @@ void plan_groups(rt_grid g, bool strict = false) {
   split_last_wave(g);
 }
 
+void free_table(rt_grid g) {
+  if (g->wt) cudaFree(g->wt);   // (waits for the sweeps that read it)
+  g->wt = nullptr;
+  g->wt_bytes = 0;
+}
+
 template <typename T>
 rt_status upload_plan(rt_grid g) {
   g->gen++;
+  if (!g->stream && !(sizeof(T) == 8 && g->variant == 1 && g->interp == RT_INTERP_LINEAR)) free_table(g);
   std::vector<AngleParam<T>> ap(g->group_angles.size());
   for (size_t gi = 0; gi < g->groups.size(); ++gi) {
     const GroupParam &gp = g->groups[gi];
@@ -1051,9 +1058,7 @@ rt_status ensure_seg_table(rt_grid g, cudaStream_t s) {
   const size_t need = g->stream ? stream_table_bytes(g) : 2 * slots * (size_t)N_of(g) * sizeof(T);
   if (need > g->wt_bytes) {
     const bool room = table_room(g, need);
-    if (g->wt) cudaFree(g->wt);
-    g->wt = nullptr;
-    g->wt_bytes = 0;
+    free_table(g);
     if (!room || cudaMalloc(&g->wt, need) != cudaSuccess) {
       cudaGetLastError();
       g->wt = nullptr;
@@ -1963,11 +1968,7 @@ rt_status rt_set_table_limit(rt_grid g, long long bytes) {
   if (bytes < -1) return fail(RT_ERR_ARG, "the table limit must be >= 0, or -1 for automatic");
   cudaStreamSynchronize(g->own);
   g->wt_limit = bytes;
-  if (g->wt && bytes >= 0 && g->wt_bytes > (size_t)bytes) {
-    cudaFree(g->wt);   // (waits for the sweeps that read it)
-    g->wt = nullptr;
-    g->wt_bytes = 0;
-  }
+  if (bytes >= 0 && g->wt_bytes > (size_t)bytes) free_table(g);
   g->no_stream = g->wt_off = false;   // decided again at the next solve
   plan_groups(g);
   rt_status r = upload_plan_any(g);
@@ -2336,6 +2337,7 @@ rt_status rt_set_interpolation(rt_grid g, int order) {
   plan_groups(g);
   rt_status r = upload_plan_any(g);
   if (r != RT_OK) return r;
+  if (g->first64 && order != RT_INTERP_LINEAR) free_table(g->first64);   // it iterates linear solves only
   if (g->sub64) return rt_set_interpolation(g->sub64, order);
   return RT_OK;
 }

@@ -160,6 +160,22 @@ def test_a_later_medium_finds_the_room_that_an_earlier_one_had_not(rt, prec):
     np.testing.assert_allclose(J2, J, rtol=1e-12 if prec == "fp64" else 1e-5)
 
 
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_second_order_holds_no_table(rt, prec):
+    p = W.random_box(16, 12, 8, seed=480, n_mu=4)
+    with _grid(rt, p, prec, {}, None) as g:
+        a = g.ali_solve(tol=1e-6, max_iter=200)[0], g.get_S()
+        assert g.sweep_table()["bytes"] > 0
+        g.set_interpolation("quadratic")
+        assert g.sweep_table()["bytes"] == 0
+        g.ali_solve(tol=1e-6, max_iter=20, raise_on_fail=False)
+        assert g.sweep_table()["bytes"] == 0
+        g.set_interpolation("linear")
+        b = g.ali_solve(tol=1e-6, max_iter=200)[0], g.get_S()
+        assert a[0] == b[0] and g.sweep_table()["bytes"] > 0
+        np.testing.assert_array_equal(a[1], b[1])
+
+
 def test_fp64_tables_of_unpadded_rows(rt):
     """Rows of one cell: the streamed sweep's table (rows padded to 16 bytes) is twice
     as large as the one-cell-per-thread sweep's, which fits the limit alone."""
