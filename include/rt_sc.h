@@ -374,7 +374,8 @@ rt_status rt_set_sweep_config(rt_grid g, int angles_per_group, int cluster_ctas,
  * is planned without it (variant 3 then is the pipelined sweep), until a medium is
  * set while there is room or the limit is set again.  Also applies to
  * a mixed grid's internal FP64 grids.  Frees a table that is too large now and
- * replans the sweep.  Errors: RT_ERR_ARG for bytes < -1. */
+ * replans the sweep.  A grid gives its tables back by itself, until the next medium,
+ * where an allocation of its own finds no memory.  Errors: RT_ERR_ARG for bytes < -1. */
 rt_status rt_set_table_limit(rt_grid g, long long bytes);
 
 /* Whether the sweep as planned reads its weights from the table (*streams 1 or 0;

@@ -902,12 +902,37 @@ rt_status upload_plan_any(rt_grid g) {
   return g->desc.prec == RT_PREC_FP64 ? upload_plan<double>(g) : upload_plan<float>(g);
 }
 
+// Gives back the tables of a grid and its internal grids, which are planned without
+// until a later medium: what a solve or its moments cannot do without goes first.
+// False if there was none to give (or the new plan could not be set up).
+bool shed_tables(rt_grid g) {
+  bool any = false;
+  cudaGetLastError();
+  for (rt_grid h : {g, g->first64, g->sub64}) {
+    if (!h || !h->wt) continue;
+    free_table(h);
+    h->no_stream = h->wt_off = true;
+    plan_groups(h);
+    if (upload_plan_any(h) != RT_OK) return false;
+    any = true;
+  }
+  return any;
+}
+
+rt_status grid_malloc(rt_grid g, void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && shed_tables(g)) e = cudaMalloc(p, bytes);
+  CU(e);
+  return RT_OK;
+}
+
 rt_status ensure_tmp(rt_grid g, size_t n) {
   if (n <= g->tmp_n) return RT_OK;
   if (g->tmp) cudaFree(g->tmp);
   g->tmp = nullptr;
   g->tmp_n = 0;
-  CU(cudaMalloc((void **)&g->tmp, n * sizeof(double)));
+  rt_status r = grid_malloc(g, (void **)&g->tmp, n * sizeof(double));
+  if (r != RT_OK) return r;
   g->tmp_n = n;
   return RT_OK;
 }
@@ -1334,8 +1359,12 @@ rt_status ali_loop(rt_grid g, const rt_solve_opts *opts, cudaStream_t s, int *it
     if (r != RT_OK) return r;
   }
   if (gs) {
-    const long long gen = g->gen;
+    long long gen = g->gen;
     rt_status r = gs_setup<T>(g, s, incremental != 0, GA);
+    if (r == RT_ERR_OOM && shed_tables(g)) {
+      gen = g->gen;
+      r = gs_setup<T>(g, s, incremental != 0, GA);
+    }
     if (r != RT_OK) return r;
     if (g->wt_gen == gen) g->wt_gen = g->gen;   // new buffers of its own leave the table as it was
   }
@@ -1568,11 +1597,17 @@ template <typename T>
 rt_status moments_sweep(rt_grid g, cudaStream_t s) {
   rt_status r0 = ensure_seg_table<T>(g, s);
   if (r0 != RT_OK) return r0;
-  const size_t need = g->groups.size();
-  if (need > g->mpart_groups) {
+  while (g->groups.size() > g->mpart_groups) {
+    const size_t need = g->groups.size();
     if (g->Mpart) cudaFree(g->Mpart);
     g->Mpart = nullptr;
-    CU(cudaMalloc(&g->Mpart, need * 9 * (size_t)N_of(g) * sizeof(T)));
+    g->mpart_groups = 0;
+    const cudaError_t e = cudaMalloc(&g->Mpart, need * 9 * (size_t)N_of(g) * sizeof(T));
+    if (e == cudaErrorMemoryAllocation && shed_tables(g)) {   // (another plan: other groups)
+      if ((r0 = ensure_seg_table<T>(g, s)) != RT_OK) return r0;
+      continue;
+    }
+    CU(e);
     g->mpart_groups = need;
   }
   rtk::SweepArgs<T> A = sweep_args<T>(g);
@@ -1588,7 +1623,8 @@ rt_status ensure_tmp2(rt_grid g, size_t n) {
   if (g->tmp2) cudaFree(g->tmp2);
   g->tmp2 = nullptr;
   g->tmp2_n = 0;
-  CU(cudaMalloc((void **)&g->tmp2, n * sizeof(double)));
+  rt_status r = grid_malloc(g, (void **)&g->tmp2, n * sizeof(double));
+  if (r != RT_OK) return r;
   g->tmp2_n = n;
   return RT_OK;
 }
@@ -2042,7 +2078,11 @@ rt_status rt_set_opacity_source(rt_grid g, const double *chi_tot, const double *
   if ((r = init_ghosts_any(g, g->S, s)) != RT_OK) return r;
   for (int f = 0; f < 6; ++f)
     if ((r = fill_bc_any(g, f, s)) != RT_OK) return r;
-  if (g->desc.prec == RT_PREC_MIXED && ((r = plan_first64(g)) != RT_OK || (r = plan_bins(g)) != RT_OK)) return r;
+  if (g->desc.prec == RT_PREC_MIXED) {
+    auto internal_grids = [&] { return (r = plan_first64(g)) == RT_OK ? plan_bins(g) : r; };
+    if ((r = internal_grids()) == RT_ERR_OOM && shed_tables(g)) r = internal_grids();
+    if (r != RT_OK) return r;
+  }
   g->gs_ready = false;
   g->gen++;
   g->have_medium = true;

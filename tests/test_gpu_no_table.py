@@ -160,6 +160,25 @@ def test_a_later_medium_finds_the_room_that_an_earlier_one_had_not(rt, prec):
     np.testing.assert_allclose(J2, J, rtol=1e-12 if prec == "fp64" else 1e-5)
 
 
+def test_tables_give_way_to_what_the_moments_need(rt):
+    """With 1.16 GB free and no table but the FP64 iterations' (0.27 GB) the moments'
+    0.87 GB fit; a float32 table of 0.13 GB must not take their place."""
+    p = W.random_box(128, 128, 128, seed=490, n_mu=2)
+    with _grid(rt, p, "mixed", dict(angles_per_group=1), None) as g:
+        g.ali_solve(tol=1e-6, max_iter=5, raise_on_fail=False)
+        want = g.moments(want=("J", "K"))
+    with _grid(rt, p, "mixed", dict(angles_per_group=1), None) as g:
+        with free_memory_of(1160 << 20):
+            g.ali_solve(tol=1e-6, max_iter=5, raise_on_fail=False)
+            assert g.sweep_table()["bytes"] == (8 + 16) * 8 * 128 ** 3
+            got = g.moments(want=("J", "K"))
+            assert g.sweep_table()["bytes"] == 0
+            g.ali_solve(tol=1e-6, max_iter=5, raise_on_fail=False)
+            again = g.moments(want=("J", "K"))
+    for m in (got, again):
+        assert rel(m["J"], want["J"]) < 1e-5 and rel(m["K"][:, :3], want["K"][:, :3]) < 1e-5
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_second_order_holds_no_table(rt, prec):
     p = W.random_box(16, 12, 8, seed=480, n_mu=4)
