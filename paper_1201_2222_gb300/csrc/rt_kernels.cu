@@ -1879,14 +1879,15 @@ constexpr int kMomentSplitBlocks = 608;   // up to so many tiles
 template <typename T>
 __global__ void __launch_bounds__(kAliTile * kAliRows, 4) reduce_moments_kernel(Dims d, int ngroups, int nxg, const T *Jpart,
                                                                              const T *Mpart, double *J, double *H,
-                                                                             double *K, double *F, int two_d, int parts) {
+                                                                             double *K, double *F, int two_d, int parts,
+                                                                             int f0) {
   constexpr int KR = kAliTile / kAliRows;
   __shared__ double tile[kAliTile][kAliTile + 1];
   const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
   const int tx = threadIdx.x % kAliTile, ty = threadIdx.x / kAliTile;
   const int tiles_x = (nx + kAliTile - 1) / kAliTile;
   const int x0 = (blockIdx.x % tiles_x) * kAliTile, y0 = (blockIdx.x / tiles_x) * kAliTile;
-  const int z = blockIdx.y, f = blockIdx.z / parts, part = blockIdx.z % parts;
+  const int z = blockIdx.y, f = f0 + blockIdx.z / parts, part = blockIdx.z % parts;
   const long long cells = d.cells, N = cells * d.nf, fb = f * cells;
   const int x = x0 + tx;
   double s[KR];
@@ -2296,9 +2297,11 @@ cudaError_t launch_reduce_moments(const Dims &d, int ngroups, int nxg, const T *
                                   double *H, double *K, double *F, int two_d, cudaStream_t s) {
   const int tiles = ((d.n[0] + kAliTile - 1) / kAliTile) * ((d.n[1] + kAliTile - 1) / kAliTile);
   const int parts = (long long)tiles * d.n[2] * d.nf <= kMomentSplitBlocks ? 3 : 1;
-  const dim3 grid((unsigned)tiles, (unsigned)d.n[2], (unsigned)(d.nf * parts));
-  reduce_moments_kernel<T><<<grid, kAliTile * kAliRows, 0, s>>>(d, ngroups, nxg, Jpart, Mpart, J, H, K, F, two_d,
-                                                                parts);
+  for (int f0 = 0; f0 < d.nf; f0 += 65535) {   // (a grid's z extent; three parts only where nf is small)
+    const dim3 grid((unsigned)tiles, (unsigned)d.n[2], (unsigned)(std::min(d.nf - f0, 65535) * parts));
+    reduce_moments_kernel<T><<<grid, kAliTile * kAliRows, 0, s>>>(d, ngroups, nxg, Jpart, Mpart, J, H, K, F, two_d,
+                                                                  parts, f0);
+  }
   return cudaGetLastError();
 }
 

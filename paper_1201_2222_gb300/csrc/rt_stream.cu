@@ -837,7 +837,6 @@ template <typename T>
 __global__ void __launch_bounds__(256) stream_table_kernel(const SweepArgs<T> A, T *WT) {
   constexpr int SEG = SegOf<T>::N;
   const GroupParam gp = A.grp[blockIdx.y];
-  const int f = blockIdx.z;
   int cax[3];
   plane_axes(gp.axis, cax);
   const int Nu = pick3(A.d.n, cax[0]), Nv = pick3(A.d.n, cax[1]), Nw = pick3(A.d.n, cax[2]);
@@ -845,9 +844,10 @@ __global__ void __launch_bounds__(256) stream_table_kernel(const SweepArgs<T> A,
             perW = pick3(A.d.periodic, cax[2]);
   const int nseg = (Nu + SEG - 1) / SEG;
   const long long rows = (long long)Nv * Nw, n = rows * nseg;
-  const T *chi = A.chiP[gp.axis] + (long long)f * A.d.cells;
-  T *out = WT + (gp.a0 * (long long)A.d.nf + f) * A.wt_slot;
+  for (int f = blockIdx.z; f < A.d.nf; f += gridDim.z)
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const T *chi = A.chiP[gp.axis] + (long long)f * A.d.cells;
+    T *out = WT + (gp.a0 * (long long)A.d.nf + f) * A.wt_slot;
     const long long rw = i / nseg;
     const int u0 = (int)(i - rw * nseg) * SEG;
     const int w = (int)(rw / Nv), v = (int)(rw - (long long)w * Nv);
@@ -961,7 +961,7 @@ template <typename T>
 cudaError_t launch_stream_table(const SweepArgs<T> &A, T *WT, cudaStream_t s) {
   const long long n = A.d.cells / std::min(A.d.n[0], A.d.n[1]) * ((std::max(A.d.n[0], A.d.n[1]) + SegOf<T>::N - 1) / SegOf<T>::N);
   const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152LL * 16)), (unsigned)A.ngroups,
-                  (unsigned)A.d.nf);
+                  (unsigned)std::min(A.d.nf, 65535));
   stream_table_kernel<T><<<grid, 256, 0, s>>>(A, WT);
   return cudaGetLastError();
 }
