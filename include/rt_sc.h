@@ -254,6 +254,14 @@ rt_status rt_set_iteration(rt_grid g, int scheme);
  * to exercise the path.  Errors: RT_ERR_ARG for a negative limit. */
 rt_status rt_set_wait_limit(rt_grid g, long long polls);
 
+/* Polls (of about a microsecond at most) after which a streamed sweep's wait on the
+ * edge row of a neighbouring strip gives up (default 2^20, about a second at most).
+ * The strips of that plane then stop exchanging rows, the sweep ends, and the solve
+ * returns RT_ERR_CUDA with device error code 33; the grid stays usable.  Applies to a
+ * mixed grid's internal FP64 grids too.  No counterpart in the paper; tests set it
+ * to 0 (no wait is granted a poll).  Errors: RT_ERR_ARG for a negative limit. */
+rt_status rt_set_row_wait_limit(rt_grid g, int polls);
+
 /* Mixed grids, Jacobi ALI solves with linear interpolation: after the first
  * (FP64) iteration, another iteration is done in FP64 from the current S each
  * time the largest relative change of S (Eq. 25) has fallen by the factor

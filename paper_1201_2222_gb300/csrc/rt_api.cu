@@ -356,6 +356,7 @@ struct rt_grid_s {
   int *gs_list = nullptr;             // forward groups, then forward rays with mu_V < 0
   size_t gs_list_n = 0;
   long long gs_polls = 1LL << 22;     // polls of a reverse-phase barrier wait before it gives up
+  int row_polls = 1 << 20;            // polls of a streamed sweep's wait on a neighbouring strip
   double *gs_acc = nullptr;           // incremental solves: J of the forward and of the reverse
                                       // rays [2][nf][cells]
 
@@ -1033,6 +1034,7 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
   A.depth = g->depth;
   A.ncomp = g->ncomp;
   A.one_pass = g->one_pass;
+  A.row_polls = g->row_polls;
   const bool wt = ready && !g->stream && g->variant == 1 && g->interp == RT_INTERP_LINEAR;
   const size_t half = g->wt_bytes / 2;
   A.WE = wt ? (const T *)g->wt : nullptr;
@@ -1690,6 +1692,7 @@ rt_status plan_bins(rt_grid g) {
     if ((r = rt_set_interpolation(g->sub64, g->interp)) != RT_OK) return r;
     if ((r = rt_set_iteration(g->sub64, g->iteration)) != RT_OK) return r;
     g->sub64->wt_limit = g->wt_limit;
+    g->sub64->row_polls = g->row_polls;
     g->bins64 = ill;
   }
   const size_t C = (size_t)g->d.cells, m = ill.size();
@@ -1731,6 +1734,7 @@ rt_status plan_first64(rt_grid g) {
     if (r != RT_OK) return r;
     g->first64->shadow = true;
     g->first64->wt_limit = g->wt_limit;
+    g->first64->row_polls = g->row_polls;
     // a few FP64 iterations per solve: their segment weights are tabulated per
     // medium when the table is modest (it holds E and Psi0 of every ray and cell)
     if (2.0 * g->na * (double)N_of(g) * 8.0 > kShadowTableMax) {
@@ -2429,6 +2433,18 @@ rt_status rt_set_wait_limit(rt_grid g, long long polls) {
   if (polls < 0) return fail(RT_ERR_ARG, "the poll limit must be >= 0");
   g->gs_polls = polls;
   g->gen++;   // captured batches hold the old limit
+  return RT_OK;
+}
+
+rt_status rt_set_row_wait_limit(rt_grid g, int polls) {
+  if (!g) return fail(RT_ERR_ARG, "NULL grid");
+  if (polls < 0) return fail(RT_ERR_ARG, "the poll limit must be >= 0");
+  for (rt_grid h : {g, g->first64, g->sub64}) {
+    if (!h) continue;
+    h->row_polls = polls;
+    if (h->wt_gen == h->gen) h->wt_gen++;
+    h->gen++;   // captured batches hold the old limit (the table stays)
+  }
   return RT_OK;
 }
 

@@ -37,6 +37,7 @@ struct SweepArgs {
   int depth;                 //    planes of a CTA's S ring: 3, 4 or 6
   int ncomp;                 //    its threads with cells
   int one_pass;              //    1: a strip's row segments are at most ncomp
+  int row_polls;             //    polls before a wait on a neighbouring strip's row gives up
   int gs_forward;            // 1: Gauss-Seidel forward phase -- groups crossing the
   int gs_axis;               //    gs_axis face with mu < 0 (the reverse rays) do nothing
   // subdomain (EXTERNAL) z faces, side 0 = low, 1 = high (one-cell-per-thread

@@ -207,25 +207,30 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
 }
 
-// A word that counts bytes as they arrive (one phase a plane of its parity).  A wait
-// gives up after kArrivalPolls polls.
-constexpr int kArrivalPolls = 1 << 22;
+// A word that counts bytes as they arrive (one phase a plane of its parity).  A wait gives
+// up after `polls` polls, of about a microsecond at most, or when `lost` is set: a strip
+// that gives up sets it in every strip of its cluster, and from then on none of them
+// waits, stores into another or arms a word again; they sweep on with what they have, and
+// the solve ends in an error.  A neighbour is at most two planes ahead of the rows that a
+// strip has sent, so a word takes three rows at most beyond its last arming (3 x 37 KB of
+// its range of 1 MB).
 __device__ __forceinline__ void arrival_init(unsigned bar) {
   asm volatile("mbarrier.init.shared.b64 [%0], 1;" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrival_expect(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ bool arrival_wait(unsigned bar, unsigned parity) {
-  for (int i = 0; i < kArrivalPolls; ++i) {
+__device__ __forceinline__ bool arrival_wait(unsigned bar, unsigned parity, const int *lost, int polls) {
+  for (int i = 0; i < polls; ++i) {
     unsigned done;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 1000;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
+    if (*(const volatile int *)lost) break;
   }
   return false;
 }
@@ -250,6 +255,9 @@ __device__ __forceinline__ void st_remote(unsigned a, const double2 (&v)[1], uns
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(a), "d"(v[0].x),
                "d"(v[0].y), "r"(bar)
                : "memory");
+}
+__device__ __forceinline__ void st_flag(unsigned a) {
+  asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], 1;" ::"r"(a) : "memory");
 }
 __device__ __forceinline__ void st_remote_one(unsigned a, float v, unsigned bar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(a), "f"(v), "r"(bar) : "memory");
@@ -308,7 +316,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
   T *PU = HU + D * nU;                         // [D][nU]  ghosts that the outflow there replaces
   __shared__ RayConst<T> RC[kStreamRays];
   __shared__ unsigned long long Arr[2][2];     // arrival of the halo rows: [before, after the strip][plane parity]
-  __shared__ int lost;                         // a wait on them gave up: no more waits, nothing is re-armed
+  __shared__ int lost;                         // a wait on them gave up in this cluster
 
   const int fs = A.st->fs_count + A.parity_offset;
   const int prev = fs & 1;
@@ -629,17 +637,20 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
       bool pushTop = false, pushBot = false;
       unsigned aTop = 0, aBot = 0, bTop = 0, bBot = 0;
       if (edge) {
-        if (t > 0 && !*(volatile int *)&lost) {
+        bool dead = __any_sync(0xffffffffu, *(volatile int *)&lost);
+        if (t > 0 && !dead) {
           const unsigned bar = sArr + ((t - 1) & 1) * 8, par = ((t - 1) >> 1) & 1;
           bool ok = true;
-          if (has_top && __any_sync(0xffffffffu, lv == 0)) ok = arrival_wait(bar, par);
-          if (has_bot && __any_sync(0xffffffffu, lv == R - 1)) ok = arrival_wait(bar + 16, par) && ok;
-          if (!ok) {
+          if (has_top && __any_sync(0xffffffffu, lv == 0)) ok = arrival_wait(bar, par, &lost, A.row_polls);
+          if (has_bot && __any_sync(0xffffffffu, lv == R - 1)) ok = arrival_wait(bar + 16, par, &lost, A.row_polls) && ok;
+          dead = __any_sync(0xffffffffu, !ok);
+          if (dead) {
             *(volatile int *)&lost = 1;
-            atomicCAS(&A.st->err, 0, kStreamTimeout);
+            if (lane < C) st_flag(mapa_rank(smem_addr(&lost), lane));
+            if (lane == 0) atomicCAS(&A.st->err, 0, kStreamTimeout);
           }
         }
-        if (t + 1 < Nw) {
+        if (t + 1 < Nw && !dead) {
           pushTop = has_top && lv == 0 && base + lane < ntask;
           pushBot = has_bot && lv == R - 1 && base + lane < ntask;
           if (has_top) {
@@ -808,7 +819,13 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
       const long long off = ((long long)f * A.na + A.ang[gp.a0 + a].angle) * A.d.gsize + (long long)(v0 + row) * Nu + u;
       ghost_store<T>(Gp, Gn, Gdn, off, Il[a * pb + (row + 1) * W + X0 + u], inc, emit);
     }
-  if (C > 1) cluster.sync();   // no strip leaves while another may still store into its halo rows
+  if (C > 1) {
+    cluster.sync();   // no strip leaves while another may still store into its halo rows
+    if (*(volatile int *)&lost) {   // (in all of them or none) rows that nobody waited for may be on their way
+      for (int i = 0; i < 50; ++i) __nanosleep(1000);
+      cluster.sync();
+    }
+  }
 }
 
 template <typename T, bool MOM, bool RAG, bool ONE>

@@ -113,6 +113,7 @@ _SIGS = {
     "rt_fetch": (ctypes.c_int, [_VP, ctypes.c_longlong, _VP, _VP, _VP]),
     "rt_measure_rates": (ctypes.c_int, [_VP, ctypes.c_int]),
     "rt_set_wait_limit": (ctypes.c_int, [_VP, ctypes.c_longlong]),
+    "rt_set_row_wait_limit": (ctypes.c_int, [_VP, ctypes.c_int]),
     "rt_set_fp64_anchors": (ctypes.c_int, [_VP, ctypes.c_double]),
     "rt_set_fp64_bin_limit": (ctypes.c_int, [_VP, ctypes.c_double]),
     "rt_set_external_face": (ctypes.c_int, [_VP, ctypes.c_int, _VP, _VP, _VP, _VP, ctypes.c_int,
@@ -434,6 +435,10 @@ class Grid:
     def set_wait_limit(self, polls):
         """Polls before a Gauss-Seidel grid-barrier wait gives up (rt_set_wait_limit)."""
         _check(load().rt_set_wait_limit(self._h, int(polls)))
+
+    def set_row_wait_limit(self, polls):
+        """Polls before a streamed sweep's wait on a neighbouring strip gives up (rt_set_row_wait_limit)."""
+        _check(load().rt_set_row_wait_limit(self._h, int(polls)))
 
     def set_interpolation(self, order):
         """Face interpolation: INTERP_LINEAR / "linear" or INTERP_QUADRATIC / "quadratic"."""
