@@ -148,7 +148,8 @@ rt_status rt_set_boundary_intensity(rt_grid g, int face, const double *I);
  * S: [nf][nz][ny][nx] or NULL to use the grid's current S; when S is given the
  * periodic ghosts are reset to the image cells' S (first-iteration semantics),
  * otherwise the lagged ghosts of the previous formal solution are used and
- * advanced.  J_out, lstar_out: [nf][nz][ny][nx] or NULL.  opts may be NULL.
+ * advanced.  With on_device and a stream in opts the call returns without waiting;
+ * a device error is then reported by the next call that waits.  J_out, lstar_out: [nf][nz][ny][nx] or NULL.  opts may be NULL.
  * Errors: RT_ERR_STATE before rt_set_opacity_source. */
 rt_status rt_formal_solve(rt_grid g, const double *S, double *J_out, double *lstar_out,
                           int on_device, const rt_solve_opts *opts);
@@ -257,7 +258,9 @@ rt_status rt_set_wait_limit(rt_grid g, long long polls);
 /* Polls (of about a microsecond at most) after which a streamed sweep's wait on the
  * edge row of a neighbouring strip gives up (default 2^20, about a second at most).
  * The strips of that plane then stop exchanging rows, the sweep ends, and the solve
- * returns RT_ERR_CUDA with device error code 33; the grid stays usable.  Applies to a
+ * returns RT_ERR_CUDA with device error code 33; the grid stays usable.  (After a
+ * formal solution of device arrays on a caller's stream, which reads nothing back, it
+ * is the next call reading the solver's state that returns it.)  Applies to a
  * mixed grid's internal FP64 grids too.  No counterpart in the paper; tests set it
  * to 0 (no wait is granted a poll).  Errors: RT_ERR_ARG for a negative limit. */
 rt_status rt_set_row_wait_limit(rt_grid g, int polls);

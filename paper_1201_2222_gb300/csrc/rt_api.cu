@@ -320,6 +320,7 @@ struct rt_grid_s {
   // since the last FP64 formal solution, one more iteration in FP64 from the
   // current S, whose J replaces the accumulated one (0: none after the first)
   double anchor_drop = 1e-2;
+  rtk::SolveState *report = nullptr;  // the shadow's sweeps report their errors into its owner's state
   bool shadow = false;                // this grid is another grid's FP64 first-solution shadow
   bool stepped = false;               // an ALI solve begun by rt_ali_begin may be continued
   // Mixed grids: frequency bins too ill-conditioned for float32 even as
@@ -993,12 +994,20 @@ rt_status fill_bc_any(rt_grid g, int face, cudaStream_t s) {
   return g->desc.prec == RT_PREC_FP64 ? fill_bc<double>(g, face, s) : fill_bc<float>(g, face, s);
 }
 
-// Error word written by the bounds-checked debug build's kernels.
+// The error word of a state just read: a wait that gave up, or the bounds-checked debug
+// build's finding.  Reported once; a formal solution on a caller's stream leaves it to the
+// next call that reads the state.
+rt_status device_error(rt_grid g, const rtk::SolveState &hs) {
+  if (!hs.err) return RT_OK;
+  CU(cudaMemset(&g->st->err, 0, sizeof(int)));
+  CU(cudaMemset(&g->st->err_info, 0, sizeof(int)));
+  CU(cudaStreamSynchronize(nullptr));
+  return fail(RT_ERR_CUDA, "device check failed (code %d, index %d)", hs.err, hs.err_info);
+}
 rt_status check_device_error(rt_grid g) {
   rtk::SolveState hs{};
   CU(cudaMemcpy(&hs, g->st, sizeof hs, cudaMemcpyDeviceToHost));
-  if (hs.err) return fail(RT_ERR_CUDA, "device check failed (code %d, index %d)", hs.err, hs.err_info);
-  return RT_OK;
+  return device_error(g, hs);
 }
 
 template <typename T>
@@ -1024,6 +1033,7 @@ rtk::SweepArgs<T> sweep_args(rt_grid g) {
   A.Opart = g->interp == RT_INTERP_QUADRATIC ? (T *)g->Opart : nullptr;
   A.Mpart = (T *)g->Mpart;
   A.st = g->st;
+  A.err = &(g->report ? g->report : g->st)->err;
   A.parity_offset = 0;
   A.write_ghosts = 1;
   A.skip_if_done = 1;
@@ -1479,7 +1489,7 @@ rt_status ali_loop(rt_grid g, const rt_solve_opts *opts, cudaStream_t s, int *it
     enqueued += m;
     CU(cudaMemcpyAsync(&hs, g->st, sizeof hs, cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    if (hs.err) return fail(RT_ERR_CUDA, "device check failed (code %d, index %d)", hs.err, hs.err_info);
+    if (hs.err) return device_error(g, hs);
     if (hs.done || enqueued >= max_iter) break;
     if (fp64_its && g->anchor_drop > 0.0) {
       if (anchor_ref < 0.0) {
@@ -1549,7 +1559,7 @@ rt_status ali_iterate(rt_grid g, int n, cudaStream_t s, int *iters, double *resi
   rtk::SolveState hs{};
   CU(cudaMemcpyAsync(&hs, g->st, sizeof hs, cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
-  if (hs.err) return fail(RT_ERR_CUDA, "device check failed (code %d, index %d)", hs.err, hs.err_info);
+  if (hs.err) return device_error(g, hs);
   if (iters) *iters = hs.iter;
   if (resid) *resid = hs.last_resid;
   g->fs_total = hs.fs_count;
@@ -1733,6 +1743,7 @@ rt_status plan_first64(rt_grid g) {
     rt_status r = rt_create_grid(&d, &g->first64);
     if (r != RT_OK) return r;
     g->first64->shadow = true;
+    g->first64->report = g->st;
     g->first64->wt_limit = g->wt_limit;
     g->first64->row_polls = g->row_polls;
     // a few FP64 iterations per solve: their segment weights are tabulated per
@@ -2147,6 +2158,7 @@ rt_status rt_formal_solve(rt_grid g, const double *S, double *J_out, double *lst
     o2.stream = (void *)s;
     if ((r = rt_formal_solve(g->sub64, Ssub, tj, tl, 1, &o2)) != RT_OK) return r;
     CU(cudaStreamSynchronize(s));
+    if ((r = check_device_error(g->sub64)) != RT_OK) return r;
     if ((r = move_bins(g->bins64, tj, g->J, C, false, cudaMemcpyDeviceToDevice, s)) != RT_OK) return r;
     if ((r = move_bins(g->bins64, tl, g->lstar, C, false, cudaMemcpyDeviceToDevice, s)) != RT_OK) return r;
   }
@@ -2857,7 +2869,7 @@ rt_status ls_step(rt_lockstep L, std::vector<LsResult> *done) {
     bool finished = true;
     rt_status st = RT_OK;
     if (hs.err) {
-      st = fail(RT_ERR_CUDA, "device check failed (code %d, index %d)", hs.err, hs.err_info);
+      st = device_error(g, hs);
     } else if (!(hs.done || x->enqueued >= x->max_iter)) {
       finished = false;
       if (x->fp64_its && g->anchor_drop > 0.0) {

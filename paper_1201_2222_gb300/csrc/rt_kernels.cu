@@ -1641,7 +1641,9 @@ __global__ void finish_kernel(SolveState *st) {
   st->fs_count += 1;
   st->iter += 1;
   st->last_resid = r;
-  if (r <= st->tol) {
+  if (st->err) {             // the host reports it; what is enqueued behind does nothing
+    st->done = 1;
+  } else if (r <= st->tol) {
     st->done = 1;
     st->converged = 1;
   } else if (st->iter >= st->max_iter) {
@@ -1651,9 +1653,7 @@ __global__ void finish_kernel(SolveState *st) {
 
 // Small state edits, in stream order.
 __global__ void state_op_kernel(SolveState *st, int op, int a, double b, int c) {
-  if (op == 0) {           // reset for a new ALI solve (and its error word)
-    st->err = 0;
-    st->err_info = 0;
+  if (op == 0) {           // reset for a new ALI solve (the error word stays until the host has reported it)
     st->fs_count = 0;
     st->iter = 0;
     st->done = 0;

@@ -23,6 +23,7 @@ struct SweepArgs {
   T *Opart;                  // second-order sweeps: sum_k w_k (1 - dI0/dS0) per group, same layout
   T *Mpart;                  // [ngroups][9][nf][cells] (moments launches only)
   SolveState *st;
+  int *err;                  // error word that a streamed sweep reports into: of the grid whose status is read
   int parity_offset;         // ghost parity = (st->fs_count + parity_offset) & 1
   int write_ghosts;
   int skip_if_done;

@@ -282,7 +282,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
   const GroupParam gp = A.grp[gi];
   if (A.gs_forward && gp.axis == A.gs_axis && gp.sa < 0) return;   // swept in the reverse phase
   if (gp.na > A.ray_slots) {   // plan inconsistent with the shared-memory layout: refuse to run
-    if (threadIdx.x == 0) atomicCAS(&A.st->err, 0, 32);
+    if (threadIdx.x == 0) atomicCAS(A.err, 0, 32);
     return;
   }
   int cax[3];
@@ -647,7 +647,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
           if (dead) {
             *(volatile int *)&lost = 1;
             if (lane < C) st_flag(mapa_rank(smem_addr(&lost), lane));
-            if (lane == 0) atomicCAS(&A.st->err, 0, kStreamTimeout);
+            if (lane == 0) atomicCAS(A.err, 0, kStreamTimeout);
           }
         }
         if (t + 1 < Nw && !dead) {

@@ -51,3 +51,32 @@ def test_a_wait_that_runs_out(rt, prec, shape, strips):
         with pytest.raises(rt.RTError) as e:
             g.set_row_wait_limit(-1)
         assert e.value.status == rt.RT_ERR_ARG
+
+
+def test_a_lost_row_of_a_formal_solution_on_a_stream_is_reported_later(rt):
+    p = W.random_box(24, 20, 12, seed=530, n_mu=6, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    with _grid(rt, p, "fp64", cluster_ctas=4, variant=3) as g:
+        g.set_row_wait_limit(0)
+        B = torch.from_numpy(p.B).cuda()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(torch.cuda.Stream()):
+            g.formal_solve(B)                               # returns without reading the state
+        g.set_row_wait_limit(1 << 20)
+        with pytest.raises(rt.RTError) as e:
+            g.ali_solve(tol=1e-6, max_iter=20)
+        assert e.value.status == rt.RT_ERR_CUDA and "code 33" in str(e.value)
+        g.ali_solve(tol=1e-6, max_iter=20, raise_on_fail=False)
+
+
+def test_a_lost_row_of_the_fp64_iterations_is_reported(rt):
+    """A solve of one iteration, which a mixed grid does on its internal FP64 grid (planes
+    of 96 x 96 cells, several strips)."""
+    p = W.random_box(96, 96, 96, seed=540, n_mu=6, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    with _grid(rt, p, "mixed") as g:
+        g.set_row_wait_limit(0)
+        with pytest.raises(rt.RTError) as e:
+            g.ali_solve(tol=1e-6, max_iter=1)
+        assert e.value.status == rt.RT_ERR_CUDA and "code 33" in str(e.value)
+        g.set_row_wait_limit(1 << 20)
+        it, _, st = g.ali_solve(tol=1e-6, max_iter=1, raise_on_fail=False)
+        assert it == 1 and st == rt.RT_ERR_NOT_CONVERGED
