@@ -1724,6 +1724,57 @@ rt_status plan_bins(rt_grid g) {
   return RT_OK;
 }
 
+// The host side of a grid with this description (angle set, sizes, rays): false for an
+// n_mu without angle set.
+bool describe(rt_grid g, const rt_grid_desc &D) {
+  g->desc = D;
+  g->two_d = D.nz == 1;
+  if (g->two_d) {   // z-invariant: the z faces are never crossed; treat z as periodic
+    g->desc.bc_lo[2] = g->desc.bc_hi[2] = RT_BC_PERIODIC;
+    g->desc.dz = 1.0;
+  }
+  if (!level_symmetric(D.n_mu, g->two_d, g->mu, g->wq)) return false;
+  g->na = (int)g->wq.size();
+  g->tsize = D.prec == RT_PREC_FP64 ? 8 : 4;
+  rtk::Dims &d = g->d;
+  d.n[0] = D.nx;
+  d.n[1] = D.ny;
+  d.n[2] = D.nz;
+  d.nf = D.nfreq;
+  d.cells = (long long)D.nx * D.ny * D.nz;
+  for (int a = 0; a < 3; ++a) {
+    d.bc_lo[a] = g->desc.bc_lo[a];
+    d.bc_hi[a] = g->desc.bc_hi[a];
+    d.periodic[a] = g->desc.bc_lo[a] == RT_BC_PERIODIC;
+  }
+  d.face[0] = (long long)D.nz * D.ny;
+  d.face[1] = (long long)D.nz * D.nx;
+  d.face[2] = (long long)D.ny * D.nx;
+  d.gsize = d.face[0] + d.face[1] + d.face[2];
+  build_rays(g);
+  return true;
+}
+
+// Groups per frequency of a grid with this description: of its automatic plans, with and
+// without the weight table, but at least those of two rays where the rays allow (a tuned
+// plan); every ray its own where no device can be asked what is resident.
+long long most_groups(const rt_grid_desc &D, long long na) {
+  int dev = 0;
+  if (cudaGetDeviceCount(&dev) != cudaSuccess || dev < 1 || !(D.dx > 0) || !(D.dy > 0) || (D.nz > 1 && !(D.dz > 0))) {
+    cudaGetLastError();
+    return na;
+  }
+  size_t most = (size_t)(na + 1) / 2 + 6;
+  for (bool table : {true, false}) {
+    rt_grid_s g;
+    g.wt_never = !table;
+    describe(&g, D);
+    plan_groups(&g);
+    most = std::max(most, g.groups.size());
+  }
+  return (long long)most;
+}
+
 // Mixed grids: the internal FP64 grid that does the first formal solution of
 // each Jacobi ALI solve with linear interpolation (not needed when every eps = 1,
 // whose solves only iterate the boundary ghosts).
@@ -1802,34 +1853,11 @@ rt_status rt_create_grid(const rt_grid_desc *desc, rt_grid *out) {
         return fail(RT_ERR_ARG, "subdomain z faces do not combine with fixed x or y faces");
   }
   rt_grid g = new rt_grid_s();
-  g->desc = D;
-  g->two_d = D.nz == 1;
-  if (g->two_d) {   // z-invariant: the z faces are never crossed; treat z as periodic
-    g->desc.bc_lo[2] = g->desc.bc_hi[2] = RT_BC_PERIODIC;
-    g->desc.dz = 1.0;
-  }
-  if (!level_symmetric(D.n_mu, g->two_d, g->mu, g->wq)) {
+  if (!describe(g, D)) {
     delete g;
     return fail(RT_ERR_ARG, "n_mu must be 2, 4, 6, 8, 10 or 12 (got %d)", D.n_mu);
   }
-  g->na = (int)g->wq.size();
-  g->tsize = D.prec == RT_PREC_FP64 ? 8 : 4;
-  rtk::Dims &d = g->d;
-  d.n[0] = D.nx;
-  d.n[1] = D.ny;
-  d.n[2] = D.nz;
-  d.nf = D.nfreq;
-  d.cells = (long long)D.nx * D.ny * D.nz;
-  for (int a = 0; a < 3; ++a) {
-    d.bc_lo[a] = g->desc.bc_lo[a];
-    d.bc_hi[a] = g->desc.bc_hi[a];
-    d.periodic[a] = g->desc.bc_lo[a] == RT_BC_PERIODIC;
-  }
-  d.face[0] = (long long)D.nz * D.ny;
-  d.face[1] = (long long)D.nz * D.nx;
-  d.face[2] = (long long)D.ny * D.nx;
-  d.gsize = d.face[0] + d.face[1] + d.face[2];
-  build_rays(g);
+  const rtk::Dims &d = g->d;
   plan_groups(g);
 
   auto cleanup = [&](rt_status st) {
@@ -1945,7 +1973,7 @@ rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
   const long long na = (long long)q.size();
   const long long cells = (long long)D.nx * D.ny * D.nz;
   const long long gsize = (long long)D.nx * D.ny + (long long)D.ny * D.nz + (long long)D.nx * D.nz;
-  const long long groups = (na + 1) / 2 + 6;   // the planner groups at least two rays where it can
+  const long long groups = most_groups(D, na);
   const long long N = cells * D.nfreq;
   const long long ts = D.prec == RT_PREC_FP64 ? 8 : 4;
   long long b = 8 * N * (D.prec == RT_PREC_MIXED ? 13 : 11)   // FP64 fields and state
@@ -1959,7 +1987,9 @@ rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
   // a mixed grid's internal FP64 grid for its FP64 iterations: fields, FP64
   // copies, ghosts, J partials (no moments pass, no table)
   if (D.prec == RT_PREC_MIXED) {
-    b += 8 * N * 11 + 8 * N * 6 + 6 * D.nfreq * na * gsize * 8 + groups * N * 8;
+    rt_grid_desc H = D;
+    H.prec = RT_PREC_FP64;
+    b += 8 * N * 11 + 8 * N * 6 + 6 * D.nfreq * na * gsize * 8 + most_groups(H, na) * N * 8;
     if (2.0 * na * (double)N * 8.0 <= kShadowTableMax) b += 2 * na * pad * D.nfreq * 8;   // its segment-weight table
   }
   *bytes = b;
@@ -3081,31 +3111,7 @@ extern "C" rt_status rt_formal_solve_noalloc(const rt_grid_desc *desc, const dou
   // the size limit is checked before any pointer is touched
   rt_grid_s g;
   g.wt_never = true;   // no segment-weight table: this entry point allocates nothing
-  g.desc = D;
-  g.two_d = D.nz == 1;
-  if (g.two_d) {
-    g.desc.bc_lo[2] = g.desc.bc_hi[2] = RT_BC_PERIODIC;
-    g.desc.dz = 1.0;
-  }
-  if (!level_symmetric(D.n_mu, g.two_d, g.mu, g.wq))
-    return fail(RT_ERR_ARG, "n_mu must be 2, 4, 6, 8, 10 or 12 (got %d)", D.n_mu);
-  g.na = (int)g.wq.size();
-  g.tsize = D.prec == RT_PREC_FP64 ? 8 : 4;
-  g.d.n[0] = D.nx;
-  g.d.n[1] = D.ny;
-  g.d.n[2] = D.nz;
-  g.d.nf = D.nfreq;
-  g.d.cells = (long long)D.nx * D.ny * D.nz;
-  for (int a = 0; a < 3; ++a) {
-    g.d.bc_lo[a] = g.desc.bc_lo[a];
-    g.d.bc_hi[a] = g.desc.bc_hi[a];
-    g.d.periodic[a] = g.desc.bc_lo[a] == RT_BC_PERIODIC;
-  }
-  g.d.face[0] = (long long)D.nz * D.ny;
-  g.d.face[1] = (long long)D.nz * D.nx;
-  g.d.face[2] = (long long)D.ny * D.nx;
-  g.d.gsize = g.d.face[0] + g.d.face[1] + g.d.face[2];
-  build_rays(&g);
+  if (!describe(&g, D)) return fail(RT_ERR_ARG, "n_mu must be 2, 4, 6, 8, 10 or 12 (got %d)", D.n_mu);
   plan_groups(&g);
   cudaStream_t s = (cudaStream_t)stream;
   return D.prec == RT_PREC_FP64 ? noalloc_run<double>(g, chi, S, B, J_out, s)
