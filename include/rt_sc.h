@@ -487,8 +487,10 @@ typedef struct {
   long long footprint;      /* estimated device bytes */
 } rt_request_info;
 
-/* Estimated device memory of a grid with this description (upper bound of the
- * arrays it allocates, with the moments pass; for RT_PREC_MIXED including the
+/* Estimated device memory of a grid with this description, linear interpolation, the
+ * Jacobi iteration and an automatic or tuned sweep plan (upper bound of the
+ * arrays it allocates, with the moments pass and the table of segment weights where
+ * it streams; the server counts second-order and Gauss-Seidel requests as such; for RT_PREC_MIXED including the
  * internal FP64 grid of its FP64 iterations, but not the FP64 grid of ill-
  * conditioned bins that some media add: up to an RT_PREC_FP64 grid of those
  * bins, see RT_PREC_MIXED).  Errors: RT_ERR_ARG. */

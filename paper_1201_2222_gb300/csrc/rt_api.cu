@@ -1757,20 +1757,25 @@ bool describe(rt_grid g, const rt_grid_desc &D) {
 
 // Groups per frequency of a grid with this description: of its automatic plans, with and
 // without the weight table, but at least those of two rays where the rays allow (a tuned
-// plan); every ray its own where no device can be asked what is resident.
-long long most_groups(const rt_grid_desc &D, long long na) {
+// plan); every ray its own where no device can be asked what is resident.  The bytes of
+// the table of segment weights: 0 for a grid that never streams.
+long long most_groups(const rt_grid_desc &D, int interp, int iteration, long long na, long long *table_bytes) {
+  *table_bytes = 0;
+  if (!(D.dx > 0) || !(D.dy > 0) || (D.nz > 1 && !(D.dz > 0))) return na;   // (no grid can be made of it)
   int dev = 0;
-  if (cudaGetDeviceCount(&dev) != cudaSuccess || dev < 1 || !(D.dx > 0) || !(D.dy > 0) || (D.nz > 1 && !(D.dz > 0))) {
-    cudaGetLastError();
-    return na;
-  }
+  const bool host = cudaGetDeviceCount(&dev) != cudaSuccess || dev < 1;
+  if (host) cudaGetLastError();
   size_t most = (size_t)(na + 1) / 2 + 6;
   for (bool table : {true, false}) {
     rt_grid_s g;
     g.wt_never = !table;
+    g.interp = interp;
+    g.iteration = iteration;
     describe(&g, D);
-    plan_groups(&g);
-    most = std::max(most, g.groups.size());
+    if (!host) plan_groups(&g);
+    most = std::max(most, host ? (size_t)na : g.groups.size());
+    if (table && (host ? interp == RT_INTERP_LINEAR && !external_faces(&g) : g.stream))
+      *table_bytes = (long long)stream_table_bytes(&g);
   }
   return (long long)most;
 }
@@ -1965,6 +1970,12 @@ rt_status rt_destroy_grid(rt_grid g) {
 int rt_num_angles(rt_grid g) { return g ? g->na : 0; }
 
 rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
+  return grid_footprint(desc, RT_INTERP_LINEAR, RT_ITER_JACOBI, bytes);
+}
+
+}  // extern "C"
+
+rt_status grid_footprint(const rt_grid_desc *desc, int interp, int iteration, long long *bytes) {
   if (!desc || !bytes) return fail(RT_ERR_ARG, "rt_grid_footprint: NULL argument");
   const rt_grid_desc &D = *desc;
   if (D.nx < 1 || D.ny < 1 || D.nz < 1 || D.nfreq < 1) return fail(RT_ERR_ARG, "grid sizes and nfreq must be >= 1");
@@ -1973,7 +1984,8 @@ rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
   const long long na = (long long)q.size();
   const long long cells = (long long)D.nx * D.ny * D.nz;
   const long long gsize = (long long)D.nx * D.ny + (long long)D.ny * D.nz + (long long)D.nx * D.nz;
-  const long long groups = most_groups(D, na);
+  long long table = 0, table64 = 0;
+  const long long groups = most_groups(D, interp, iteration, na, &table);
   const long long N = cells * D.nfreq;
   const long long ts = D.prec == RT_PREC_FP64 ? 8 : 4;
   long long b = 8 * N * (D.prec == RT_PREC_MIXED ? 13 : 11)   // FP64 fields and state
@@ -1981,20 +1993,22 @@ rt_status rt_grid_footprint(const rt_grid_desc *desc, long long *bytes) {
               + 6 * D.nfreq * na * gsize * ts  // ghosts (two parities, increments) and inflow faces
               + groups * N * ts * 11           // J, Lambda* and moment partials
               + 8 * (16 * N + cells);          // moments outputs
-  // tabulated segment weights: two values per ray and cell, rows padded to 16 bytes
-  const long long pad = std::max({(D.nx + 3) / 4 * 4 * (long long)D.ny * D.nz, D.nx * ((D.ny + 3) / 4 * 4LL) * D.nz});
-  b += 2 * na * pad * D.nfreq * ts;
+  b += table;
+  if (iteration == RT_ITER_GAUSS_SEIDEL)   // correction weights, J of forward and reverse rays, the reverse phase's planes
+    b += 8 * N * 11 + 4 * D.nfreq * na * gsize * ts;
   // a mixed grid's internal FP64 grid for its FP64 iterations: fields, FP64
-  // copies, ghosts, J partials (no moments pass, no table)
+  // copies, ghosts, J partials (no moments pass), and their table
   if (D.prec == RT_PREC_MIXED) {
     rt_grid_desc H = D;
     H.prec = RT_PREC_FP64;
-    b += 8 * N * 11 + 8 * N * 6 + 6 * D.nfreq * na * gsize * 8 + most_groups(H, na) * N * 8;
-    if (2.0 * na * (double)N * 8.0 <= kShadowTableMax) b += 2 * na * pad * D.nfreq * 8;   // its segment-weight table
+    b += 8 * N * 11 + 8 * N * 6 + 6 * D.nfreq * na * gsize * 8 + most_groups(H, interp, RT_ITER_JACOBI, na, &table64) * N * 8;
+    if (2.0 * na * (double)N * 8.0 <= kShadowTableMax && iteration == RT_ITER_JACOBI) b += table64;
   }
   *bytes = b;
   return RT_OK;
 }
+
+extern "C" {
 
 int rt_angle_table(int n_mu, int two_d, double *mu, double *w) {
   std::vector<double> m, q;

@@ -22,6 +22,9 @@ struct LsResult {
   std::string message;   // the error message when status != RT_OK
 };
 
+// rt_grid_footprint of a grid set to this interpolation order and iteration scheme.
+rt_status grid_footprint(const rt_grid_desc *desc, int interp, int iteration, long long *bytes);
+
 rt_status ls_create(cudaStream_t s, rt_lockstep *out);
 void ls_destroy(rt_lockstep L);
 // Begins the solve of g (as rt_ali_solve with S = B would) and adds it.

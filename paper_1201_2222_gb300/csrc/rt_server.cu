@@ -373,18 +373,19 @@ rt_status rt_server_destroy(rt_server s) {
 rt_status rt_submit(rt_server s, const rt_request *req, long long *id_out) {
   if (!s || !req || !id_out || !req->chi || !req->eps || !req->B)
     return rt_internal_error(RT_ERR_ARG, "rt_submit: NULL argument");
-  long long fp = 0;
-  rt_status st = rt_grid_footprint(&req->desc, &fp);
-  if (st != RT_OK) return st;
   if (req->interp != 0 && req->interp != RT_INTERP_LINEAR && req->interp != RT_INTERP_QUADRATIC)
     return rt_internal_error(RT_ERR_ARG, "rt_submit: interp must be 0, 1 or 2");
   if (req->iteration != RT_ITER_JACOBI && req->iteration != RT_ITER_GAUSS_SEIDEL)
     return rt_internal_error(RT_ERR_ARG, "rt_submit: iteration must be 0 or 1");
   if (req->iteration == RT_ITER_GAUSS_SEIDEL && req->interp == RT_INTERP_QUADRATIC)
     return rt_internal_error(RT_ERR_ARG, "rt_submit: the Gauss-Seidel iteration takes linear interpolation");
+  const int interp = req->interp == 0 ? RT_INTERP_LINEAR : req->interp;
+  long long fp = 0;
+  rt_status st = grid_footprint(&req->desc, interp, req->iteration, &fp);
+  if (st != RT_OK) return st;
   Request *r = new Request();
   r->desc = req->desc;
-  r->interp = req->interp == 0 ? RT_INTERP_LINEAR : req->interp;
+  r->interp = interp;
   const size_t N = (size_t)req->desc.nx * req->desc.ny * req->desc.nz * req->desc.nfreq;
   r->chi.assign(req->chi, req->chi + N);
   r->eps.assign(req->eps, req->eps + N);

@@ -36,3 +36,22 @@ def test_many_rays(rt, prec, table, shape, n_mu):
         groups, tables = g.sweep_plan()["groups"], g.sweep_table()["bytes"]
     least = groups * N * ts * 10 + 128 * N + tables + (8 * 13 + 8 * 17 if prec == "mixed" else 8 * 11) * N
     assert rt.grid_footprint(p, prec) >= least
+
+
+def test_only_grids_that_stream_count_a_table(rt):
+    """A second-order request holds no table (2 x 4 bytes per ray and cell, 2 x 8 of the
+    FP64 iterations' grid), nor does a subdomain (2 x 8)."""
+    p = W.random_box(32, 32, 32, seed=610, n_mu=8, eps_range=(0.3, 1.0))
+    N, na = p.chi.size, 80
+    srv = rt.Server(workers=1)
+    fp = {}
+    for interp in ("linear", "quadratic"):
+        i = srv.submit(p, prec="mixed", interp=interp, tol=1e-3)
+        fp[interp] = srv.wait(i)["footprint"]
+        srv.fetch(i)
+    srv.close()
+    assert fp["linear"] == rt.grid_footprint(p)
+    assert fp["quadratic"] <= fp["linear"] - 0.95 * 24 * na * N
+    q = W.random_box(32, 32, 32, seed=610, n_mu=8, bc_lo=(P, P, X), bc_hi=(P, P, X))
+    r = W.random_box(32, 32, 32, seed=610, n_mu=8, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    assert rt.grid_footprint(q, "fp64") <= rt.grid_footprint(r, "fp64") - 0.95 * 16 * na * N
