@@ -51,17 +51,18 @@ TOL = 1e-6
 FLOPS_PER_UPDATE = 34
 # special-function results per update: the exponential and the reciprocal of dtau
 MUFU_PER_UPDATE = 2
+# the streamed sweep reads E and Psi0 (8 bytes an update in float32) and is left with two
+# interpolants (S-, I-: 14), I0 = S- + E (I- - S-) + Psi0 (S0 - S-) (2 subtractions,
+# 2 multiplies, 2 adds) and the J accumulation (2), and no special function
+STREAM_FLOPS_PER_UPDATE = 22
+STREAM_BYTES_PER_UPDATE = 8
 # CTAs per cluster of every grid in the request server's shared-launch mode
 SHARED_CLUSTER = 4
 
 # DRAM read + write bytes per launch of the sweep kernel from an ncu capture of
 # the same workload and plan (None when none was taken for the plan in use, or
 # the kernel has changed since); keyed by workload, plan, shared-memory size and groups
-PROFILED_TRAFFIC = {
-    # one launch of the 256^3 x 48-ray solve's sweep (dram__bytes_read.sum +
-    # dram__bytes_write.sum, one ncu pass)
-    ("stratified_turbulent_256^3_lq6", 3, 2, 16, 512, 197312, 27): 1235145216 + 1810619648,
-}
+PROFILED_TRAFFIC = {}
 
 
 def profiled_traffic(plan, p):
@@ -70,9 +71,13 @@ def profiled_traffic(plan, p):
     return PROFILED_TRAFFIC.get(key)
 
 
-# sweep kernel of each planner variant (simple, tiled, pipelined)
+# sweep kernel of each planner variant (simple, tiled, pipelined) without the weight table
 SWEEP_KERNEL_NAMES = {1: "sc_sweep_kernel<float>", 2: "sc_sweep_tiled_kernel<float>",
                       3: "sc_sweep_pipe_kernel<float>"}
+
+
+def sweep_kernel_name(plan, streams):
+    return "sc_sweep_stream_kernel<float>" if streams else SWEEP_KERNEL_NAMES[plan["variant"]]
 
 
 def workload():
@@ -215,19 +220,26 @@ def run_reference(args):
 
 # ------------------------------------------------------------------ GPU arm
 
-def sweep_roofline(stats_list, p, rates):
+def sweep_roofline(stats_list, p, rates, streams):
     """Roofline of the formal-solution kernel from the sweep launches timed inside
-    the solves (CUDA events on the launching stream)."""
+    the solves (CUDA events on the launching stream): the operations that the kernel
+    does, and the rate of its other stream, the tabulated weights or the special
+    functions."""
     sweep_ms = sum(s["sweep_ms"] for s in stats_list)
     sweep_n = sum(s["sweep_launches"] for s in stats_list)
     per_launch_upd = p.cells * p.n_angles * p.nf
     avg_s = (sweep_ms / sweep_n) / 1e3 if sweep_n else float("nan")
-    achieved = FLOPS_PER_UPDATE * per_launch_upd / avg_s / 1e12
+    flops = STREAM_FLOPS_PER_UPDATE if streams else FLOPS_PER_UPDATE
+    achieved = flops * per_launch_upd / avg_s / 1e12
     peak = max(rates["fp32_fma_flops"], rates["fp32x2_fma_flops"]) / 1e12
     mufu_peak = min(rates["mufu_ex2_per_s"], rates["mufu_rcp_per_s"])
-    return {"avg_launch_ms": avg_s * 1e3, "launches": sweep_n, "achieved": achieved, "peak": peak,
-            "frac": achieved / peak, "updates_per_s": per_launch_upd / avg_s,
-            "mufu_frac": MUFU_PER_UPDATE * per_launch_upd / avg_s / mufu_peak}
+    out = {"avg_launch_ms": avg_s * 1e3, "launches": sweep_n, "achieved": achieved, "peak": peak,
+           "frac": achieved / peak, "updates_per_s": per_launch_upd / avg_s, "flops_per_update": flops}
+    if streams:
+        out["weights_gbs"] = STREAM_BYTES_PER_UPDATE * per_launch_upd / avg_s / 1e9
+    else:
+        out["mufu_frac"] = MUFU_PER_UPDATE * per_launch_upd / avg_s / mufu_peak
+    return out
 
 
 def solve_rate(rt, p, prec, dev, n=2, tol=None, autotune=True):
@@ -250,9 +262,9 @@ def solve_rate(rt, p, prec, dev, n=2, tol=None, autotune=True):
     g.enable_timing(True)
     g.ali_solve(tol=tol, max_iter=20000)
     st = g.stats()
-    plan = g.sweep_plan()
+    plan, streams = g.sweep_plan(), g.sweep_table()["streams"]
     g.close()
-    return {"workload": p.name, "iters": it, "ms_per_solve": 1e3 * dt, "solves_per_s": 1.0 / dt,
+    return {"workload": p.name, "streams": streams, "iters": it, "ms_per_solve": 1e3 * dt, "solves_per_s": 1.0 / dt,
             "updates_per_s": p.cells * p.n_angles * p.nf * it / dt, "plan": plan, "stats": st}
 
 
@@ -327,7 +339,8 @@ def run_gpu(args):
     upd_local = float(sum(s["updates"] for _, _, s in rec))
     t_max, upd_all = reduce_max_sum(t_local, upd_local, dist)
     iters = [i for i, _, _ in rec]
-    roof = sweep_roofline([s for _, _, s in rec], p, rates)
+    streams = g.sweep_table()["streams"]
+    roof = sweep_roofline([s for _, _, s in rec], p, rates, streams)
 
     # end to end through the C ABI with host buffers (copies inside the timed region)
     e2e_t = []
@@ -363,7 +376,7 @@ def run_gpu(args):
         # the 128^3 periodic turbulent box (80 rays): mixed, and the plain FP64 path
         pb = W.turbulent_box(128, n_mu=8, tol=TOL)
         box = solve_rate(rt, pb, rt.MIXED, dev)
-        box["roofline"] = sweep_roofline([box.pop("stats")], pb, rates)
+        box["roofline"] = sweep_roofline([box.pop("stats")], pb, rates, box["streams"])
         extras["turbulent_box_128"] = box
         b64 = solve_rate(rt, pb, rt.FP64, dev, n=1)
         b64.pop("stats")
@@ -373,7 +386,7 @@ def run_gpu(args):
         # the 64^3 atmosphere with 64 frequency bins (all bins in one launch)
         pm = W.multifrequency_atmosphere(64, nf=64)
         mf = solve_rate(rt, pm, rt.MIXED, dev, n=1)
-        mf["roofline"] = sweep_roofline([mf.pop("stats")], pm, rates)
+        mf["roofline"] = sweep_roofline([mf.pop("stats")], pm, rates, mf["streams"])
         extras["multifrequency_64_64bins"] = mf
     if not args.skip_extras and not args.skip_gs:
         # the Gauss-Seidel scheme against Jacobi on the stratified scattering
@@ -439,14 +452,14 @@ def run_gpu(args):
         "latency_ms": {"p50": lat[len(lat) // 2], "p99": lat[min(len(lat) - 1, int(math.ceil(0.99 * len(lat))) - 1)]},
         "ali_iterations": iters[0] if len(set(iters)) == 1 else iters,
         "sweep_plan": plan,
-        "roofline": {"bound": "alu", "kernel": SWEEP_KERNEL_NAMES[plan["variant"]],
+        "roofline": {"bound": "latency" if streams else "alu", "kernel": sweep_kernel_name(plan, streams),
                      "achieved": roof["achieved"], "peak": roof["peak"], "unit": "TFLOP/s",
                      "frac": roof["frac"], "traffic": profiled_traffic(plan, p),
                      "peak_source": "measured on this GPU by rt_measure_rates: the larger of its scalar "
                                     "and packed-pair FP32 FMA rates (of measured)",
-                     "flops_per_update": FLOPS_PER_UPDATE, "avg_launch_ms": roof["avg_launch_ms"],
+                     "flops_per_update": roof["flops_per_update"], "avg_launch_ms": roof["avg_launch_ms"],
                      "launches": roof["launches"], "sweep_updates_per_s": roof["updates_per_s"],
-                     "mufu_frac": roof["mufu_frac"]},
+                     **{k: roof[k] for k in ("weights_gbs", "mufu_frac") if k in roof}},
         "measured_peaks": dict(rates, sm_count=sm_count),
         "cpu_baseline": cpu,
         "e2e": e2e,
