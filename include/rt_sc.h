@@ -324,7 +324,8 @@ rt_status rt_get_face_intensity(rt_grid g, int side, double *I, int on_device, c
  * iterations since rt_ali_begin and the max relative change of the last one
  * (Eq. 25; of J when every eps = 1).  Jacobi iteration only.  Errors:
  * RT_ERR_STATE before rt_set_opacity_source, for a Gauss-Seidel grid, or when
- * another solve or formal solution has run since rt_ali_begin. */
+ * another solve or formal solution has run, or a device error was returned, since
+ * rt_ali_begin. */
 rt_status rt_ali_begin(rt_grid g, const double *S_init, int on_device, const rt_solve_opts *opts);
 rt_status rt_ali_iterate(rt_grid g, int n, const rt_solve_opts *opts, int *iters_out, double *resid_out);
 

@@ -1559,7 +1559,10 @@ rt_status ali_iterate(rt_grid g, int n, cudaStream_t s, int *iters, double *resi
   rtk::SolveState hs{};
   CU(cudaMemcpyAsync(&hs, g->st, sizeof hs, cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
-  if (hs.err) return device_error(g, hs);
+  if (hs.err) {
+    g->stepped = false;   // the error ended this solve (its later launches would do nothing)
+    return device_error(g, hs);
+  }
   if (iters) *iters = hs.iter;
   if (resid) *resid = hs.last_resid;
   g->fs_total = hs.fs_count;

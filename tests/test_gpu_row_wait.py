@@ -80,3 +80,24 @@ def test_a_lost_row_of_the_fp64_iterations_is_reported(rt):
         g.set_row_wait_limit(1 << 20)
         it, _, st = g.ali_solve(tol=1e-6, max_iter=1, raise_on_fail=False)
         assert it == 1 and st == rt.RT_ERR_NOT_CONVERGED
+
+
+def test_a_stepped_solve_that_lost_a_row_must_begin_again(rt):
+    p = W.random_box(24, 20, 12, seed=550, n_mu=6, bc_lo=(P, P, T), bc_hi=(P, P, V))
+    with _grid(rt, p, "fp64", cluster_ctas=4, variant=3) as g:
+        g.ali_begin()
+        g.ali_iterate(2)
+        g.set_row_wait_limit(0)
+        with pytest.raises(rt.RTError) as e:
+            g.ali_iterate(2)
+        assert e.value.status == rt.RT_ERR_CUDA and "code 33" in str(e.value)
+        g.set_row_wait_limit(1 << 20)
+        with pytest.raises(rt.RTError) as e:
+            g.ali_iterate(2)
+        assert e.value.status == rt.RT_ERR_STATE
+        g.ali_begin()
+        a = g.ali_iterate(3)
+        with _grid(rt, p, "fp64", cluster_ctas=4, variant=3) as fresh:
+            fresh.ali_begin()
+            assert fresh.ali_iterate(3) == a
+            np.testing.assert_array_equal(g.get_S(), fresh.get_S())
