@@ -48,6 +48,8 @@ rt_status fail(rt_status st, const char *fmt, ...) {
   vsnprintf(buf, sizeof buf, fmt, ap);
   va_end(ap);
   g_err = buf;
+  // reported here: a later launch must not find the runtime's record of it
+  if (st == RT_ERR_OOM || st == RT_ERR_CUDA) cudaGetLastError();
   return st;
 }
 
