@@ -255,8 +255,8 @@ rt_status rt_set_iteration(rt_grid g, int scheme);
  * to exercise the path.  Errors: RT_ERR_ARG for a negative limit. */
 rt_status rt_set_wait_limit(rt_grid g, long long polls);
 
-/* Polls (of about a microsecond at most) after which a streamed sweep's wait on the
- * edge row of a neighbouring strip gives up (default 2^20, about a second at most).
+/* Polls (of about 0.1 ms at most) after which a streamed sweep's wait on the edge row
+ * of a neighbouring strip gives up (default 2^13, about a second at most).
  * The strips of that plane then stop exchanging rows, the sweep ends, and the solve
  * returns RT_ERR_CUDA with device error code 33; the grid stays usable.  (After a
  * formal solution of device arrays on a caller's stream, which reads nothing back, it

@@ -359,7 +359,7 @@ struct rt_grid_s {
   int *gs_list = nullptr;             // forward groups, then forward rays with mu_V < 0
   size_t gs_list_n = 0;
   long long gs_polls = 1LL << 22;     // polls of a reverse-phase barrier wait before it gives up
-  int row_polls = 1 << 20;            // polls of a streamed sweep's wait on a neighbouring strip
+  int row_polls = 1 << 13;            // polls of a streamed sweep's wait on a neighbouring strip
   double *gs_acc = nullptr;           // incremental solves: J of the forward and of the reverse
                                       // rays [2][nf][cells]
 

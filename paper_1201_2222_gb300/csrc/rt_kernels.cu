@@ -1636,17 +1636,16 @@ __global__ void inv_denominator_kernel(long long n, const double *eps, const dou
 // Convergence decision after one ALI iteration (single thread).
 __global__ void finish_kernel(SolveState *st) {
   if (st->done) return;
+  const int err = st->err;   // the host reports it; what is enqueued behind does nothing
   const double r = __longlong_as_double((long long)st->resid_bits);
   st->resid_bits = 0ULL;
   st->fs_count += 1;
   st->iter += 1;
   st->last_resid = r;
-  if (st->err) {             // the host reports it; what is enqueued behind does nothing
-    st->done = 1;
-  } else if (r <= st->tol) {
+  if (r <= st->tol) {
     st->done = 1;
     st->converged = 1;
-  } else if (st->iter >= st->max_iter) {
+  } else if (err || st->iter >= st->max_iter) {
     st->done = 1;
   }
 }

@@ -29,7 +29,8 @@
 // per warp and segment of 4 cells against about 260 in the pipelined sweep, which
 // forms the weights as it goes.  One sweep, CUDA events, before (the pipelined or
 // one-cell-per-thread sweep with its best or automatic plan) and now:
-//   float32  128^3 x 80 rays  0.90 / 1.52 ms -> 0.55     256^3 x 48  5.83 -> 3.4
+//   float32  128^3 x 80 rays  0.90 / 1.52 ms -> 0.55     256^3 x 48  5.83 -> 3.85
+//            (automatic plan; 3.4 with 3 rays and 16 strips)
 //            512 x 512 x 4 bins x 24 rays  2.16 -> 0.85
 //   float64  96^3 x 48 rays  2.13 ms -> 1.39 (the FP64 pipe alone: 0.88)
 #include <cooperative_groups.h>
@@ -208,7 +209,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
 }
 
 // A word that counts bytes as they arrive (one phase a plane of its parity).  A wait gives
-// up after `polls` polls, of about a microsecond at most, or when `lost` is set: a strip
+// up after `polls` polls, of about 0.1 ms at most, or when `lost` is set: a strip
 // that gives up sets it in every strip of its cluster, and from then on none of them
 // waits, stores into another or arms a word again; they sweep on with what they have, and
 // the solve ends in an error.  A neighbour is at most two planes ahead of the rows that a
@@ -224,7 +225,7 @@ __device__ __forceinline__ bool arrival_wait(unsigned bar, unsigned parity, cons
   for (int i = 0; i < polls; ++i) {
     unsigned done;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 100000;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
@@ -265,6 +266,17 @@ __device__ __forceinline__ void st_remote_one(unsigned a, float v, unsigned bar)
 __device__ __forceinline__ void st_remote_one(unsigned a, double v, unsigned bar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(a), "d"(v), "r"(bar) : "memory");
 }
+
+// The strip of this thread lost a row: told to the C strips of its cluster.  As a call
+// where a thread keeps one segment of whole rows: the inlined code costs that sweep
+// registers (2D, 512 x 512 x 4 bins: 100.5 ms a solve inlined, 89.5 as a call; the others
+// lose 1 % by a call).
+__device__ __forceinline__ void give_up(int *lost, int C, int *err) {
+  *(volatile int *)lost = 1;
+  for (int r = 0; r < C; ++r) st_flag(mapa_rank(smem_addr(lost), r));
+  atomicCAS(err, 0, kStreamTimeout);
+}
+__device__ __noinline__ void give_up_call(int *lost, int C, int *err) { give_up(lost, C, err); }
 
 // One cluster's (group, frequency) instance of the grid described by A.  RAG: some
 // sweep axis has rows that are no multiple of a segment; ONE: a strip's segments are
@@ -316,7 +328,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
   T *PU = HU + D * nU;                         // [D][nU]  ghosts that the outflow there replaces
   __shared__ RayConst<T> RC[kStreamRays];
   __shared__ unsigned long long Arr[2][2];     // arrival of the halo rows: [before, after the strip][plane parity]
-  __shared__ int lost;                         // a wait on them gave up in this cluster
+  __shared__ alignas(8) int lost[2];           // [0]: a wait on them gave up in this cluster; [1]: polls of a wait
 
   const int fs = A.st->fs_count + A.parity_offset;
   const int prev = fs & 1;
@@ -347,7 +359,8 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
     RC[tid] = c;
   }
   if (tid == 0 && C > 1) {
-    lost = 0;
+    lost[0] = 0;
+    lost[1] = A.row_polls;
     for (int i = 0; i < 4; ++i) arrival_init(smem_addr(&Arr[i >> 1][i & 1]));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -637,20 +650,19 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
       bool pushTop = false, pushBot = false;
       unsigned aTop = 0, aBot = 0, bTop = 0, bBot = 0;
       if (edge) {
-        bool dead = __any_sync(0xffffffffu, *(volatile int *)&lost);
-        if (t > 0 && !dead) {
+        int flag, polls;                                 // (one load: the limit's own would cost a plane 1 %)
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(flag), "=r"(polls) : "r"(smem_addr(lost)));
+        bool live = !flag;
+        if (t > 0 && live) {   // (the tasks of the last row and of the one before it: rows 0 and R - 1 of the strip)
           const unsigned bar = sArr + ((t - 1) & 1) * 8, par = ((t - 1) >> 1) & 1;
-          bool ok = true;
-          if (has_top && __any_sync(0xffffffffu, lv == 0)) ok = arrival_wait(bar, par, &lost, A.row_polls);
-          if (has_bot && __any_sync(0xffffffffu, lv == R - 1)) ok = arrival_wait(bar + 16, par, &lost, A.row_polls) && ok;
-          dead = __any_sync(0xffffffffu, !ok);
-          if (dead) {
-            *(volatile int *)&lost = 1;
-            if (lane < C) st_flag(mapa_rank(smem_addr(&lost), lane));
-            if (lane == 0) atomicCAS(A.err, 0, kStreamTimeout);
+          if (has_top && base + 31 >= ntask - nseg) live = arrival_wait(bar, par, lost, polls);
+          if (has_bot && (R == 1 || base < ntask - nseg)) live = arrival_wait(bar + 16, par, lost, polls) && live;
+          if (!live) {
+            if constexpr (ONE && !RAG) give_up_call(lost, C, A.err);
+            else give_up(lost, C, A.err);
           }
         }
-        if (t + 1 < Nw && !dead) {
+        if (t + 1 < Nw && live) {
           pushTop = has_top && lv == 0 && base + lane < ntask;
           pushBot = has_bot && lv == R - 1 && base + lane < ntask;
           if (has_top) {
@@ -803,7 +815,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
     if (base0 >= ntask) cp_async_commit();
     wait_groups(ahead - 1);                              // what the next plane needs is here
     __syncthreads();
-    if (C > 1 && tid == 0 && t > 0 && !*(volatile int *)&lost)   // (everybody has seen the rows of plane t - 1)
+    if (C > 1 && tid == 0 && t > 0 && !*(volatile int *)lost)   // (everybody has seen the rows of plane t - 1)
       for (int i = 0; i < 2; ++i)
         if (i ? has_bot : has_top) arrival_expect(sArr + i * 16 + ((t - 1) & 1) * 8, rowB);
     slp = sl;
@@ -821,7 +833,7 @@ __device__ __forceinline__ void stream_body(const SweepArgs<T> &A, const int ins
     }
   if (C > 1) {
     cluster.sync();   // no strip leaves while another may still store into its halo rows
-    if (*(volatile int *)&lost) {   // (in all of them or none) rows that nobody waited for may be on their way
+    if (*(volatile int *)lost) {   // (in all of them or none) rows that nobody waited for may be on their way
       for (int i = 0; i < 50; ++i) __nanosleep(1000);
       cluster.sync();
     }
