@@ -172,10 +172,10 @@ rt_status rt_ali_solve(rt_grid g, const double *S_init, int on_device, const rt_
 /* The Jacobi ALI solves (Eqs. 24-25) of n grids together, each from S = B with
  * the same iterates, results and iteration count as rt_ali_solve would give it
  * (bit for bit), with the sweeps of grids that can share a launch merged: every
- * iteration, one launch sweeps all grids with the pipelined sweep (variant 3:
- * the mixed default) of the same precision and cluster size (rt_set_sweep_config
- * sets it; rows of a multiple of 4 cells or not) -- up to 24 grids per launch --
- * and the other grids' sweeps are launched one by one; then each grid's update.
+ * iteration, one launch sweeps all grids of variant 3 (the mixed default) of the
+ * same precision and cluster size (rt_set_sweep_config sets it), with the weight
+ * table or without, and the same kind of rows (whole 16-byte segments or not) -- up
+ * to 24 grids per launch -- and the other grids' sweeps are launched one by one; then each grid's update.
  * Grids leave as they finish; each keeps its own host-check schedule (as in
  * rt_ali_solve).  All work runs on opts->stream (NULL: the first grid's own
  * stream).  opts (may be NULL) applies to every grid.  iters, resid, status:
@@ -364,7 +364,8 @@ rt_status rt_get_stats(rt_grid g, rt_stats *out);
  * variants 2 and 3) and the kernel variant (1 = one cell per thread with direct
  * loads, 2 = shared-memory staged planes with four cells per thread,
  * 3 = pipelined: chi and S staged one plane ahead by asynchronous copies, strip
- * edges exchanged through distributed shared memory).  Automatic choice:
+ * edges exchanged through distributed shared memory; rt_get_sweep_table tells
+ * whether the streamed sweep takes its place).  Automatic choice:
  * variant 3 for RT_PREC_MIXED, 1 for FP64; rays per group and strips from the
  * runtime's count of co-resident clusters and a cost model (rt_autotune measures
  * instead).  Variant 3, and FP64's automatic choice, take the segment weights
@@ -449,7 +450,8 @@ rt_status rt_formal_solve_noalloc(const rt_grid_desc *desc, const double *chi, c
  * worker's own CUDA stream, solves, takes J, S and Q back to host memory and
  * frees the grid.  Solves on different workers overlap on the GPU; each result
  * is the same as that of the same solve run alone (deterministic kernels and a
- * plan that depends on the problem only; in the shared mode, alone with the
+ * plan that depends on the problem only, and on whether its weight table finds
+ * room, see rt_set_sweep_config; in the shared mode, alone with the
  * plan the server gives it: its cluster size set by rt_set_sweep_config, or
  * its own plan in the largest size class).  All calls are
  * thread-safe. */
